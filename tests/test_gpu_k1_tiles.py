@@ -1,0 +1,80 @@
+"""The tensor-core PartialReduce at the edges of its work split: one or two
+query halves per tile (M around multiples of 8 and 128), the two bin grids (N
+a multiple of L or not, T + 1 crossing a group of 16 grid rows), virtual bins
+(few bins folded over L), every K-loop mode, both bin maps -- against scores of
+the same stored values in 64 bits."""
+import pytest
+import torch
+
+from paper_2206_14286_gb300 import search as S
+from tests.gpu_util import ensure_built
+
+pytestmark = pytest.mark.gpu
+
+
+def scores64(d, q, dtype):
+    """FP64 scores of the values the contraction saw, and the natural scale."""
+    D = d.D
+    if dtype == "bf16":
+        xs = d.lp.view(torch.bfloat16).view(d.N, d.pitch)[:, :D].double()
+        qs = q.to(torch.bfloat16).double()
+    else:
+        s = d.scale.double()[:, None]
+        xs = d.lp.view(torch.float8_e4m3fn).view(d.N, d.pitch)[:, :D].float().double() * s
+        # the kernel leaves the per-query scale out of the value
+        # (a true division: by a Python number torch multiplies by its inverse)
+        qsc = q.abs().amax(1, keepdim=True) / torch.full((q.shape[0], 1), 448.0, device="cuda")
+        qs = (q / qsc).to(torch.float8_e4m3fn).double()
+    s = qs @ xs.t()
+    if d.metric == "l2":
+        s = s - 0.5 * (xs * xs).sum(1)[None, :]
+    scale = qs.norm(dim=1)[:, None] * xs.norm(dim=1).max()
+    if d.metric == "l2":
+        scale = scale + 0.5 * (xs * xs).sum(1).max()
+    return s, scale
+
+
+def bin_of(N, L, bins):
+    j = torch.arange(N, device="cuda")
+    if bins == "mod":
+        return j % L
+    q, r = N // L, N % L
+    big = r * (q + 1)
+    return torch.where(j < big, j // (q + 1), r + (j - big) // max(q, 1))
+
+
+@pytest.mark.parametrize("dtype,metric", [("bf16", "l2"), ("bf16", "ip"), ("e4m3t", "ip")])
+@pytest.mark.parametrize("M", [1, 7, 8, 9, 33, 127, 128, 129, 256, 257, 333, 513])
+@pytest.mark.parametrize("N,L,D", [
+    (4096, 16, 128),      # no ragged row, T a multiple of 16
+    (4097, 16, 128),      # a ragged row that starts a group of 16 grid rows
+    (40_011, 20, 100),    # virtual bins, odd row length
+    (30_000, 3, 16),      # very few bins
+    (12_345, 1, 64),      # one bin
+    (9_999, 1931, 40),    # fewer than 16 grid rows
+    (5_003, 605, 256),    # K loop, resident queries
+    (3_001, 77, 768),     # K loop, streamed queries (resident when few)
+])
+def test_partial_reduce_work_split(dtype, metric, M, N, L, D):
+    ensure_built()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N + 31 * M + D)
+    x = torch.randn((N, D), generator=g, device="cuda")
+    q = torch.randn((M, D), generator=g, device="cuda")
+    d = S.Database(x, metric=metric, dtype=dtype)
+    s, scale = scores64(d, q, dtype)
+    # FP32 accumulation of D exact products (tensor-core rounding toward zero:
+    # 2^-23 of the running magnitude a step) and the three-part BF16 half norm
+    tol = (D + 16) * 2.0 ** -23 * scale + (2.0 ** -20 * scale if metric == "l2" else 0.0)
+    for bins in ("mod", "contiguous"):
+        V, A = d.partial_reduce(q, L, bins=bins)
+        S.sync_status()
+        b = bin_of(N, L, bins)
+        best = torch.full((M, L), -float("inf"), dtype=torch.float64, device="cuda")
+        best.scatter_reduce_(1, b[None, :].expand(M, N), s, "amax")
+        A = A.long()
+        assert ((A >= 0) & (A < N)).all()
+        assert (b[A] == torch.arange(L, device="cuda")[None, :]).all()
+        own = s.gather(1, A)
+        assert ((V.double() - own).abs() <= tol).all()     # the value is its row's score
+        assert (best - own <= 2 * tol).all()               # and the bin's best
