@@ -1,9 +1,11 @@
 // api.cu -- the extern "C" boundary: argument checks, the bin planner
 // (Eq. 13-14), work decomposition, workspace layout and kernel launches.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <mutex>
 #include <new>
+#include <utility>
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
@@ -102,11 +104,12 @@ int64_t plan_bins(int64_t N, int K, double r, int round_to) {
 }
 
 // Tile shape of each K1 variant (BQ = 0: the row length is not supported).
-void k1_tile(int dtype, int D, int64_t M, int* BW, int* BQ) {
+// scores: the exact search's kernel, one bin per row.
+void k1_tile(int dtype, int D, int64_t M, bool scores, int* BW, int* BQ) {
   dtype = stored_dtype(dtype);
   if (dtype == KNN_F32) {
-    *BW = 64;
-    *BQ = 128;
+    *BQ = M <= 64 ? 64 : 128;
+    *BW = scores && *BQ == 128 ? 128 : 64;
   } else {
     *BW = 128;
     const int maxq = k1_tc_query_tile(dtype, D);
@@ -132,7 +135,7 @@ K1Plan make_plan(int64_t N, int64_t M, int64_t L, int D, int metric, int dtype,
   p.pitch = (int)round_up(D, 16);
   p.metric = metric;
   p.dtype = stored_dtype(dtype);  // KNN_E4M3_T runs here as KNN_E4M3 (all scales equal)
-  k1_tile(dtype, D, M, &p.BW, &p.BQ);
+  k1_tile(dtype, D, M, force_splits > 0, &p.BW, &p.BQ);
   if (p.BQ == 0) return p;
   p.g = L < p.BW ? (int)(p.BW / L) : 1;
   p.Lk = (int64_t)p.g * L;
@@ -252,7 +255,7 @@ struct SearchLayout {
   QueryBufs qb;
   bool keys64;      // K1 merges 64-bit (score, ~index) keys into one [M][L] array
   bool contiguous;  // bins are runs of consecutive rows
-  size_t off_qlp, off_qscale, off_qf32, off_part_v, off_part_a, off_cand, total;
+  size_t off_qlp, off_qscale, off_qf32, off_part_v, off_cand, total;
 };
 
 knn_status layout_search(const SearchArgs& a, SearchLayout* s) {
@@ -262,22 +265,27 @@ knn_status layout_search(const SearchArgs& a, SearchLayout* s) {
   int64_t L;
   if ((st = resolve_L(a, &L)) != KNN_OK) return st;
   s->contiguous = a.bin_map == KNN_BINS_CONTIGUOUS;
-  s->keys64 = k1_tcs_supported(a.dtype, a.D, a.metric, a.N, L);
-  if (s->contiguous && !s->keys64) return KNN_EUNSUPPORTED;
+  const bool tcs = k1_tcs_supported(a.dtype, a.D, a.metric, a.N, L);
+  s->keys64 = tcs || a.dtype == KNN_F32;
+  if (s->contiguous && !tcs) return KNN_EUNSUPPORTED;
   if (s->keys64) {
-    // K2 reads the merged [M][L] keys directly: a plan with one bin per L
-    K1Plan p{};
-    p.N = a.N;
-    p.M = a.M;
-    p.L = L;
-    p.Lk = L;
-    p.g = 1;
-    p.D = a.D;
-    p.pitch = (int)round_up(a.D, 16);
-    p.metric = a.metric;
-    p.dtype = stored_dtype(a.dtype);
-    p.nsplits = 1;
-    s->plan = p;
+    // K2 reads the merged [M][L] keys directly, whatever K1's plan
+    if (tcs) {
+      K1Plan p{};
+      p.N = a.N;
+      p.M = a.M;
+      p.L = L;
+      p.Lk = L;
+      p.g = 1;
+      p.D = a.D;
+      p.pitch = (int)round_up(a.D, 16);
+      p.metric = a.metric;
+      p.dtype = stored_dtype(a.dtype);
+      p.nsplits = 1;
+      s->plan = p;
+    } else {
+      s->plan = make_plan(a.N, a.M, L, a.D, a.metric, a.dtype, 0);
+    }
     s->Kp = kprime(a.K, a.rerank, L);
     s->qb = query_bytes(a.M, a.D, a.dtype, a.metric);
     size_t o = 0;
@@ -289,7 +297,6 @@ knn_status layout_search(const SearchArgs& a, SearchLayout* s) {
     o += s->qb.f32;
     s->off_part_v = o;
     o += al((size_t)a.M * L * 8);
-    s->off_part_a = o;
     s->off_cand = o;
     o += al((size_t)a.M * s->Kp * 8);
     s->total = o > kAlign ? o : kAlign;
@@ -309,8 +316,6 @@ knn_status layout_search(const SearchArgs& a, SearchLayout* s) {
   const size_t n = (size_t)((s->plan.atomic_merge ? 1 : s->plan.nsplits) * s->plan.M * s->plan.Lk);
   s->off_part_v = o;
   o += al(n * 4);
-  s->off_part_a = o;
-  if (a.dtype == KNN_F32) o += al(n * 4);
   s->off_cand = o;
   o += al((size_t)a.M * s->Kp * 8);
   s->total = o > kAlign ? o : kAlign;
@@ -359,12 +364,12 @@ cudaError_t prep_queries(const SearchArgs& a, const SearchLayout& s, char* ws, c
 cudaError_t run_k1(const K1Plan& p, const SearchArgs& a, const void* xlp, const float* xscale,
                    const float* hnorm, const void* qlp, const float* qscale, Partials parts,
                    cudaStream_t st) {
-  if (parts.keys64)
-    return launch_k1_tcs(p.N, p.M, p.L, p.D, p.metric, a.dtype, a.bin_map, xlp, xscale, hnorm,
-                         qlp, reinterpret_cast<unsigned long long*>(parts.v), st);
   if (a.dtype == KNN_F32)
     return launch_k1_simt(p, reinterpret_cast<const float*>(xlp), hnorm,
                           reinterpret_cast<const float*>(qlp), parts, st);
+  if (parts.keys64)
+    return launch_k1_tcs(p.N, p.M, p.L, p.D, p.metric, a.dtype, a.bin_map, xlp, xscale, hnorm,
+                         qlp, reinterpret_cast<unsigned long long*>(parts.v), st);
   return launch_k1_tc(p, xlp, xscale, hnorm, qlp, qscale, parts, st);
 }
 
@@ -387,10 +392,7 @@ knn_status search_impl(const SearchArgs& a, float* out_val, int32_t* out_idx, vo
   }
   if (e != cudaSuccess) return cuda_status(e);
   const bool k64 = s.keys64;
-  Partials parts{reinterpret_cast<float*>(ws + s.off_part_v),
-                 (a.dtype == KNN_F32 && !k64) ? reinterpret_cast<int32_t*>(ws + s.off_part_a)
-                                              : nullptr,
-                 0, s.plan.atomic_merge, k64};
+  Partials parts{reinterpret_cast<float*>(ws + s.off_part_v), 0, s.plan.atomic_merge, k64};
   const float* qscale = s.qb.scale ? reinterpret_cast<const float*>(ws + s.off_qscale) : nullptr;
   {
     ProfScope ps(1, st);
@@ -428,19 +430,24 @@ struct ExactLayout {
   int64_t Nc;
   K1Plan plan;  // for a full chunk
   QueryBufs qb;
-  size_t off_qlp, off_qscale, off_qf32, off_part_v, off_part_a, off_run, total;
+  size_t off_qlp, off_qscale, off_qf32, off_part_v, off_run, off_run2, off_cand, total;
 };
 
-constexpr int64_t kExactPartialBudget = (int64_t)1 << 26;  // entries per chunk
+// Scores of a chunk (4 bytes each). Smaller chunks would stay in L2 between
+// the contraction and the selection, but their launches and last waves cost
+// more: 100 queries on 1M x 128 rows 0.92 ms with 2^24, 0.86 with 2^25, 0.83
+// with 2^26.
+constexpr int64_t kExactPartialBudget = (int64_t)1 << 26;
 
 knn_status layout_exact(const SearchArgs& a, ExactLayout* s) {
   knn_status st = check_sizes(a.N, a.D, a.dtype, a.metric, a.M, a.K);
   if (st != KNN_OK) return st;
   int BW, BQ;
-  k1_tile(a.dtype, a.D, a.M, &BW, &BQ);
+  k1_tile(a.dtype, a.D, a.M, true, &BW, &BQ);
   if (BQ == 0) return KNN_EUNSUPPORTED;
   int64_t mq = a.M > 0 ? a.M : 1;
   int64_t nc = (kExactPartialBudget / mq) / BW * BW;
+  if (a.K <= kExactMaxK) nc = std::min(nc, exact_chunk_rows(a.K) / BW * BW);
   if (nc < BW) nc = BW;
   if (nc > a.N) nc = a.N;
   s->Nc = nc;
@@ -453,13 +460,14 @@ knn_status layout_exact(const SearchArgs& a, ExactLayout* s) {
   o += s->qb.scale;
   s->off_qf32 = o;
   o += s->qb.f32;
-  const size_t n = (size_t)(s->plan.M * s->plan.Lk);
   s->off_part_v = o;
-  o += al(n * 4);
-  s->off_part_a = o;
-  if (a.dtype == KNN_F32) o += al(n * 4);
+  o += al((size_t)s->plan.M * (size_t)round_up(s->plan.Lk, 4) * 4);
   s->off_run = o;
   o += al((size_t)a.M * a.K * 8);
+  s->off_run2 = o;
+  o += al((size_t)a.M * a.K * 8);
+  s->off_cand = o;
+  if (a.K <= kExactMaxK) o += al(exact_cand_bytes(a.M, nc, a.K));
   s->total = o > kAlign ? o : kAlign;
   return KNN_OK;
 }
@@ -486,20 +494,29 @@ knn_status exact_impl(const SearchArgs& a, float* out_val, int32_t* out_idx, voi
   if (e != cudaSuccess) return cuda_status(e);
   const float* qscale = s.qb.scale ? reinterpret_cast<const float*>(ws + s.off_qscale) : nullptr;
   uint64_t* run = reinterpret_cast<uint64_t*>(ws + s.off_run);
+  uint64_t* run2 = reinterpret_cast<uint64_t*>(ws + s.off_run2);
+  uint64_t* cand = reinterpret_cast<uint64_t*>(ws + s.off_cand);
   const int esz = knn_dtype_bytes(a.dtype);
   for (int64_t n0 = 0; n0 < a.N; n0 += s.Nc) {
     const int64_t nc = (a.N - n0) < s.Nc ? (a.N - n0) : s.Nc;
     K1Plan p = make_plan(nc, a.M, nc, a.D, a.metric, a.dtype, 1);
-    Partials parts{reinterpret_cast<float*>(ws + s.off_part_v),
-                   a.dtype == KNN_F32 ? reinterpret_cast<int32_t*>(ws + s.off_part_a) : nullptr,
-                   n0, false, false};
+    float* scores = reinterpret_cast<float*>(ws + s.off_part_v);
+    Partials parts{scores, n0, false, false};
     const char* xlp = reinterpret_cast<const char*>(a.db_lp) + (size_t)n0 * p.pitch * esz;
     const float* xs = a.db_scale ? a.db_scale + n0 : nullptr;
     const float* hn = a.db_hnorm ? a.db_hnorm + n0 : nullptr;
     e = run_k1(p, a, xlp, xs, hn, ws + s.off_qlp, qscale, parts, st);
     if (e == cudaErrorNotSupported) return KNN_EUNSUPPORTED;
     if (e != cudaSuccess) return cuda_status(e);
-    e = launch_k2(p, parts, a.K, n0 == 0 ? nullptr : run, run, st);
+    // one tile per bin: the packed words of the tensor-core kernel are the
+    // scores, in rows of Lk
+    const int64_t ld = a.dtype == KNN_F32 ? round_up(p.Lk, 4) : p.Lk;
+    if (a.K <= kExactMaxK) {
+      e = launch_exact_topk(scores, ld, a.M, nc, n0, a.K, n0 == 0 ? nullptr : run, run2, cand, st);
+      std::swap(run, run2);
+    } else {
+      e = launch_k2_scores(scores, ld, a.M, nc, n0, a.K, n0 == 0 ? nullptr : run, run, st);
+    }
     if (e != cudaSuccess) return cuda_status(e);
   }
   e = launch_k3(a.M, a.D, a.metric, run, a.K, a.K, qf32, q_stride, a.db_f32, a.db_lp,
@@ -767,10 +784,7 @@ knn_status knn_partial_reduce(const void* db_lp, const float* db_scale, const fl
   cudaError_t e = prep_queries(a, s, ws, &qf32, &q_stride, st);
   if (e != cudaSuccess) return cuda_status(e);
   const bool k64 = s.keys64;
-  Partials parts{reinterpret_cast<float*>(ws + s.off_part_v),
-                 (dtype == KNN_F32 && !k64) ? reinterpret_cast<int32_t*>(ws + s.off_part_a)
-                                            : nullptr,
-                 0, s.plan.atomic_merge, k64};
+  Partials parts{reinterpret_cast<float*>(ws + s.off_part_v), 0, s.plan.atomic_merge, k64};
   const float* qscale = s.qb.scale ? reinterpret_cast<const float*>(ws + s.off_qscale) : nullptr;
   e = run_k1(s.plan, a, db_lp, db_scale, db_hnorm, ws + s.off_qlp, qscale, parts, st);
   if (e == cudaErrorNotSupported) return KNN_EUNSUPPORTED;
@@ -840,7 +854,7 @@ knn_status knn_approx_max_k(const void* scores, int32_t score_dtype, int64_t M, 
   p.Lk = Lr;
   p.g = 1;
   p.nsplits = 1;
-  Partials parts{reinterpret_cast<float*>(G), nullptr, 0, false, true};
+  Partials parts{reinterpret_cast<float*>(G), 0, false, true};
   uint64_t* keys = reinterpret_cast<uint64_t*>(ws + al((size_t)M * Lr * 8));
   e = launch_k2(p, parts, K, nullptr, keys, st);
   if (e == cudaSuccess)
@@ -950,12 +964,10 @@ knn_status knn_shard_partial_reduce(const void* db_lp, const float* db_scale,
   cudaError_t e = prep_queries(a, s, ws, &qf32, &q_stride, st);
   if (e != cudaSuccess) return cuda_status(e);
   const bool k64 = s.keys64;
-  // pair and packed partials decode their rows with the shard's offset; the
-  // 64-bit keys hold local rows, offset when they become signed keys
-  Partials parts{reinterpret_cast<float*>(ws + s.off_part_v),
-                 (dtype == KNN_F32 && !k64) ? reinterpret_cast<int32_t*>(ws + s.off_part_a)
-                                            : nullptr,
-                 k64 ? 0 : row0, s.plan.atomic_merge, k64};
+  // packed partials decode their rows with the shard's offset; the 64-bit
+  // keys hold local rows, offset when they become signed keys
+  Partials parts{reinterpret_cast<float*>(ws + s.off_part_v), k64 ? 0 : row0,
+                 s.plan.atomic_merge, k64};
   const float* qscale = s.qb.scale ? reinterpret_cast<const float*>(ws + s.off_qscale) : nullptr;
   e = run_k1(s.plan, a, db_lp, db_scale, db_hnorm, ws + s.off_qlp, qscale, parts, st);
   if (e == cudaErrorNotSupported) return KNN_EUNSUPPORTED;
@@ -1008,7 +1020,7 @@ knn_status knn_shard_rescore(const int64_t* keys, int64_t M, int64_t L, int32_t 
   p.Lk = L;
   p.g = 1;
   p.nsplits = 1;
-  Partials parts{reinterpret_cast<float*>(G), nullptr, 0, false, true};
+  Partials parts{reinterpret_cast<float*>(G), 0, false, true};
   if (e == cudaSuccess) e = launch_k2(p, parts, Kp, nullptr, cand, st, /*sorted=*/false);
   const float* qf = q;
   int64_t q_stride = D;
@@ -1054,7 +1066,7 @@ knn_status knn_shard_finish(const int64_t* cand_keys, int64_t M, int32_t Kp, int
   p.Lk = Kp;
   p.g = 1;
   p.nsplits = 1;
-  Partials parts{reinterpret_cast<float*>(C), nullptr, 0, false, true};
+  Partials parts{reinterpret_cast<float*>(C), 0, false, true};
   if (e == cudaSuccess) e = launch_k2(p, parts, K, nullptr, top, st);
   // internal scores are larger-is-better: L2 reports the squared distance
   if (e == cudaSuccess)

@@ -160,7 +160,8 @@ __device__ __forceinline__ void cp_async_wait() {
 // The smallest k with r[k] == m (one of them is). The equalities become 1.0 or
 // 0.0 and add up powers of two, the largest for k = 0, so half of the work
 // runs on the FMA pipe (16 compares and 16 selects all ran on the ALU, the
-// pipe that bounds short bins).
+// pipe that bounds short bins: 2M x 96 E4M3 rows, L = 8192, 2000 queries, 1.085
+// against 1.026 ms a search).
 __device__ __forceinline__ int first_equal(const float (&r)[16], float m) {
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -959,7 +960,7 @@ int64_t grid_steps(int64_t N, int64_t Lv, TcsArgs* a) {
 }
 
 // How many virtual bins per bin: the grids are padded to groups of 16 bins, so
-// few bins waste MMAs (L = 20: two groups and 32 columns, 1.6x the steps).
+// few bins waste MMAs (L = 20: two groups of 16, 1.6x the steps).
 // The fold with the fewest steps, each further fold counted as one per cent
 // for its additional merges and position searches.
 int64_t pick_fold(int64_t N, int64_t L, int64_t row_bytes) {
@@ -1143,7 +1144,10 @@ cudaError_t launch_k1_tcs(int64_t N, int64_t M, int64_t L, int D, int metric, in
   // One or two query halves per tile: a step costs its halves' MMAs, so one
   // half is taken where the halves do not pair up (M <= 128, or 333 queries: 3
   // halves instead of 2 x 2). With one half every step is read from L2 for
-  // 128 queries instead of 256, counted as a tenth of its time.
+  // 128 queries instead of 256, counted as a tenth of its time. On 1M x 128 rows
+  // (L2) a search of 1, 128 and 333 queries took 61, 74 and 113 us with two
+  // halves and takes 51, 55 and 101 us; 64 queries on 4M x 768 rows 2.0 ms and
+  // 0.95 ms (6.5 TB/s).
   const int64_t sms = device_sm_count();
   int64_t kq1 = 1, parts1 = 1, spp1 = 1, groups1 = 1;
   tcs_schedule(cdiv(M, 2 * kQH), a.steps_per_q, sms, &a.kq, &a.parts, &a.steps_per_part, &a.groups);

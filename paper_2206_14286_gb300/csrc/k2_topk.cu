@@ -9,49 +9,14 @@
 // winners of one query this is a single bitonic sort of O(L log^2 L) work, the
 // paper's ExactRescoring; the same code streams the N scores of a chunked
 // exact search.
+#include <algorithm>
+
 #include "common.cuh"
 #include "kernels.h"
 
 namespace tpuknn {
 
 namespace {
-
-// Candidate b (an output bin, 0 <= b < L) of query i: the best partial over
-// every split s and fold f (K1 bins b + f*L).
-struct PairSource {
-  const float* v;
-  const int32_t* a;
-  int64_t M, Lk, L, nsplits, index_offset;
-  int g;
-  // The splits' entries are read four at a time, value and index together
-  // (both arrays are written for every entry), so with few queries a warp
-  // still has many loads in flight.
-  __device__ __forceinline__ uint64_t key(int64_t i, int64_t b) const {
-    uint64_t best = 0;
-    for (int f = 0; f < g; ++f) {
-      const int64_t b0 = i * Lk + b + (int64_t)f * L;
-      for (int64_t s0 = 0; s0 < nsplits; s0 += 4) {
-        int32_t jj[4];
-        float vv[4];
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          const bool in = s0 + u < nsplits;
-          const int64_t e = b0 + (s0 + u) * M * Lk;
-          jj[u] = in ? a[e] : -1;
-          vv[u] = in ? v[e] : 0.0f;
-        }
-#pragma unroll
-        for (int u = 0; u < 4; ++u) {
-          if (jj[u] >= 0) {
-            const uint64_t k = make_key(vv[u], (int32_t)(jj[u] + index_offset));
-            best = k > best ? k : best;
-          }
-        }
-      }
-    }
-    return best;
-  }
-};
 
 // Packed partials: a float whose low `bits` bits hold (2^bits - 1 - t_local),
 // t_local the tile ordinal inside the split; the bin's row is then
@@ -148,40 +113,6 @@ __device__ __forceinline__ void lane_keys(const Src& src, int64_t i, int lane, i
     k[r] = b < L ? src.key(i, b) : 0;
   }
 }
-// The same from per-split (value, index) partials: the splits are the outer
-// loop, so a lane has the loads of all its candidates of one split in flight
-// at once (with few queries the per-candidate loop over the splits left each
-// warp waiting on one load at a time).
-template <int KPL>
-__device__ __forceinline__ void lane_keys(const PairSource& src, int64_t i, int lane, int64_t L,
-                                          uint64_t (&k)[KPL]) {
-#pragma unroll
-  for (int r = 0; r < KPL; ++r) k[r] = 0;
-  for (int f = 0; f < src.g; ++f) {
-    for (int64_t s = 0; s < src.nsplits; ++s) {
-      const int64_t base = (s * src.M + i) * src.Lk + (int64_t)f * src.L + lane;
-#pragma unroll
-      for (int r0 = 0; r0 < KPL; r0 += 8) {
-        int32_t jj[8];
-        float vv[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const bool in = r0 + u < KPL && lane + 32 * (r0 + u) < L;
-          jj[u] = in ? src.a[base + 32 * (r0 + u)] : -1;
-          vv[u] = in ? src.v[base + 32 * (r0 + u)] : 0.0f;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          if (r0 + u < KPL && jj[u] >= 0) {
-            const uint64_t key = make_key(vv[u], (int32_t)(jj[u] + src.index_offset));
-            k[r0 + u] = key > k[r0 + u] ? key : k[r0 + u];
-          }
-        }
-      }
-    }
-  }
-}
-
 // One warp per query: lane l holds candidates l, l+32, ... (KPL of them),
 // sorted; Kp rounds each take the warp-wide maximum of the lane heads and pop
 // it from its lane. Keys are unique (distinct indices), so one lane pops.
@@ -524,6 +455,56 @@ cudaError_t run_k2_wsort(const Src& src, int64_t M, int64_t L, int Kp, uint64_t*
   return cudaGetLastError();
 }
 
+// Warp 0 of a radix-select pass: the digit where the count of the histogram's
+// bins from the top reaches `need`, the keys in the bins above it, and
+// whether every key in it is needed.
+__device__ __forceinline__ void pick_digit(const uint32_t* hist, int need, int lane, int& s_digit,
+                                           int& s_above, int& s_stop) {
+  // lane l sums bins 255-8l .. 248-8l; counts from the top by a warp scan
+  uint32_t c[8], sum = 0;
+#pragma unroll
+  for (int t = 0; t < 8; ++t) {
+    c[t] = hist[255 - 8 * lane - t];
+    sum += c[t];
+  }
+  uint32_t incl = sum;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += y;
+  }
+  const uint32_t excl = incl - sum;  // keys matching the prefix in higher bins
+  const bool mine = excl < (uint32_t)need && (uint32_t)need <= incl;
+  const unsigned who = __ballot_sync(0xffffffffu, mine);
+  if (who == 0) {
+    // fewer matching keys than needed cannot happen for need <= L
+    if (lane == 0) {
+      s_digit = 0;
+      s_above = 0;
+      s_stop = 1;
+    }
+  } else if (mine) {
+    uint32_t above = excl, ct = 0;
+    int tf = 7;
+    bool found = false;
+#pragma unroll
+    for (int t = 0; t < 8; ++t) {
+      if (!found) {
+        if (above + c[t] >= (uint32_t)need) {
+          tf = t;
+          ct = c[t];
+          found = true;
+        } else {
+          above += c[t];
+        }
+      }
+    }
+    s_digit = 255 - 8 * lane - tf;
+    s_above = (int)above;
+    s_stop = (above + ct == (uint32_t)need) ? 1 : 0;
+  }
+}
+
 // The best Kp of a query's L keys as a set, in no particular order (for the
 // re-rank, which orders its candidates itself): one CTA of 256 threads per
 // query holds the L keys in registers (KPT per thread, L <= 256 KPT) and
@@ -558,51 +539,7 @@ k2_select_kernel(Src src, int64_t L, int Kp, uint64_t* __restrict__ out_keys) {
       if ((int64_t)u * 256 + tid < L && (k[u] & mask) == prefix)
         atomicAdd(&hist[(uint32_t)(k[u] >> shift) & 255u], 1u);
     __syncthreads();
-    if (tid < 32) {
-      // lane l sums bins 255-8l .. 248-8l; counts from the top by a warp scan
-      uint32_t c[8], sum = 0;
-#pragma unroll
-      for (int t = 0; t < 8; ++t) {
-        c[t] = hist[255 - 8 * lane - t];
-        sum += c[t];
-      }
-      uint32_t incl = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      const uint32_t excl = incl - sum;  // keys matching the prefix in higher bins
-      const bool mine = excl < (uint32_t)need && (uint32_t)need <= incl;
-      const unsigned who = __ballot_sync(0xffffffffu, mine);
-      if (who == 0) {
-        // fewer matching keys than needed cannot happen for need <= L
-        if (lane == 0) {
-          s_digit = 0;
-          s_above = 0;
-          s_stop = 1;
-        }
-      } else if (mine) {
-        uint32_t above = excl, ct = 0;
-        int tf = 7;
-        bool found = false;
-#pragma unroll
-        for (int t = 0; t < 8; ++t) {
-          if (!found) {
-            if (above + c[t] >= (uint32_t)need) {
-              tf = t;
-              ct = c[t];
-              found = true;
-            } else {
-              above += c[t];
-            }
-          }
-        }
-        s_digit = 255 - 8 * lane - tf;
-        s_above = (int)above;
-        s_stop = (above + ct == (uint32_t)need) ? 1 : 0;
-      }
-    }
+    if (tid < 32) pick_digit(hist, need, lane, s_digit, s_above, s_stop);
     __syncthreads();
     prefix |= (uint64_t)s_digit << shift;
     mask |= (uint64_t)0xFF << shift;
@@ -644,6 +581,175 @@ cudaError_t run_k2_select(const Src& src, int64_t M, int64_t L, int Kp, uint64_t
   return cudaGetLastError();
 }
 
+// ---------------------------------------------------------------------------
+// Top-K of an exact search: a CTA takes the best K of up to 8192 elements of
+// one query, so that many CTAs share a query's scores (one CTA per query
+// streaming all of them left 100 queries on 100 SMs: 3.4 ms for 1M rows), and
+// a second launch takes the best K of the CTAs' and the earlier chunks' keys.
+//
+// Up to K = kThrMaxK: each of 256 threads holds 32 elements; the K-th largest
+// of the 256 threads' maxima is a lower bound of the K-th largest element, and
+// few elements beyond K reach it (about 126 for K = 100 of 8192), so those are
+// gathered and sorted, and no element is looked at more than twice: 0.18 ms
+// for 100 queries of 1M scores, K = 10, with the merge. Larger K,
+// or more elements at the bound than the buffer holds (ties): a radix select
+// over the keys, read again in every pass.
+// ---------------------------------------------------------------------------
+constexpr int kTopkElems = 8192, kTopkCap = 1024, kThrMaxK = 128;
+
+// Scores of a chunk: element e of query i as an ordered 64-bit key (0: no
+// candidate, which -inf and NaN are not). raw() is what a thread loads, with
+// no condition around it, so that its loads are all in flight together.
+struct ScoreSource {
+  const float* v;
+  int64_t ld, row0;
+  typedef float Raw;
+  __device__ __forceinline__ float raw(int64_t i, int64_t e) const { return v[i * ld + e]; }
+  static __device__ __forceinline__ uint32_t high(float s) {
+    return s > neg_inf() ? float_to_ordered(s) : 0u;
+  }
+  __device__ __forceinline__ uint64_t key(int64_t i, int64_t e) const {
+    const uint32_t h = high(raw(i, e));
+    return h ? ((uint64_t)h << 32) | (uint32_t)~(uint32_t)(row0 + e) : 0;
+  }
+};
+// The K keys of the running set (if any), then the CTAs' keys.
+struct MergeSource {
+  const uint64_t* run;
+  const uint64_t* cand;
+  int64_t nrun, ncand;  // per query
+  typedef uint32_t Raw;
+  __device__ __forceinline__ const uint64_t* at(int64_t i, int64_t e) const {
+    return e < nrun ? run + (i * nrun + e) : cand + (i * ncand + e - nrun);
+  }
+  __device__ __forceinline__ uint32_t raw(int64_t i, int64_t e) const {
+    return reinterpret_cast<const uint32_t*>(at(i, e))[1];
+  }
+  static __device__ __forceinline__ uint32_t high(uint32_t h) { return h; }
+  __device__ __forceinline__ uint64_t key(int64_t i, int64_t e) const { return *at(i, e); }
+};
+
+template <class Src>
+__global__ void __launch_bounds__(256)
+block_topk_kernel(Src src, int64_t n, int64_t nblk, int K, uint64_t* __restrict__ out) {
+  constexpr int KPT = kTopkElems / 256;
+  __shared__ uint64_t buf[kTopkCap];
+  __shared__ uint32_t s_mx[256];
+  __shared__ int s_cnt, s_digit, s_above, s_stop;
+  const int tid = threadIdx.x, lane = tid & 31;
+  const int64_t i = blockIdx.x / nblk, blk = blockIdx.x % nblk;
+  const int64_t e0 = blk * kTopkElems;
+  const int m = (int)min((int64_t)kTopkElems, n - e0);  // elements of this CTA
+  uint64_t* o = out + (i * nblk + blk) * K;
+  if (tid == 0) s_cnt = 0;
+  bool overflow = K > kThrMaxK;
+  if (!overflow) {
+    typename Src::Raw raw[KPT];
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) raw[u] = src.raw(i, e0 + min(u * 256 + tid, m - 1));
+    uint32_t h[KPT], mx = 0;
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) {
+      h[u] = u * 256 + tid < m ? Src::high(raw[u]) : 0u;
+      mx = max(mx, h[u]);
+    }
+    // descending sort of the 256 maxima: bitonic, one per thread
+    uint32_t x = mx;
+#pragma unroll
+    for (int size = 2; size <= 256; size <<= 1) {
+#pragma unroll
+      for (int stride = size >> 1; stride > 0; stride >>= 1) {
+        uint32_t y;
+        if (stride >= 32) {
+          __syncthreads();
+          s_mx[tid] = x;
+          __syncthreads();
+          y = s_mx[tid ^ stride];
+        } else {
+          y = __shfl_xor_sync(0xffffffffu, x, stride);
+        }
+        const bool keep_max = ((tid & stride) == 0) == ((tid & size) == 0);
+        x = keep_max ? max(x, y) : min(x, y);
+      }
+    }
+    __syncthreads();
+    s_mx[tid] = x;
+    __syncthreads();
+    const uint32_t thr = max(s_mx[K - 1], 1u);
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) {
+      if (h[u] >= thr) {
+        const int p = atomicAdd(&s_cnt, 1);
+        if (p < kTopkCap) buf[p] = src.key(i, e0 + u * 256 + tid);
+      }
+    }
+    __syncthreads();
+    overflow = s_cnt > kTopkCap;
+  }
+  if (!overflow) {
+    const int c = s_cnt;
+    if (c <= 32) {
+      if (tid >= 32) return;
+      uint64_t x = lane < c ? buf[lane] : 0;
+#pragma unroll
+      for (int size = 2; size <= 32; size <<= 1) {
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+          const uint64_t y = shfl_xor_u64(x, stride);
+          const bool keep_max = ((lane & stride) == 0) == ((lane & size) == 0);
+          x = keep_max ? (y > x ? y : x) : (y < x ? y : x);
+        }
+      }
+      for (int t = lane; t < K; t += 32) o[t] = t < 32 ? x : 0;
+      return;
+    }
+    const int P2 = next_pow2(c);
+    for (int t = c + tid; t < P2; t += 256) buf[t] = 0;
+    bitonic_sort_desc(buf, P2);
+    for (int t = tid; t < K; t += 256) o[t] = t < P2 ? buf[t] : 0;
+    return;
+  }
+  // radix select, 8 bits per pass from the top, over the keys in memory
+  uint32_t* hist = s_mx;
+  uint64_t prefix = 0, mask = 0;
+  int need = min(K, m);
+  for (int shift = 56; shift >= 0; shift -= 8) {
+    __syncthreads();
+    hist[tid] = 0;
+    __syncthreads();
+    for (int e = tid; e < m; e += 256) {
+      const uint64_t k = src.key(i, e0 + e);
+      if ((k & mask) == prefix) atomicAdd(&hist[(uint32_t)(k >> shift) & 255u], 1u);
+    }
+    __syncthreads();
+    if (tid < 32) pick_digit(hist, need, lane, s_digit, s_above, s_stop);
+    __syncthreads();
+    prefix |= (uint64_t)s_digit << shift;
+    mask |= (uint64_t)0xFF << shift;
+    need -= s_above;
+    if (s_stop) break;
+  }
+  // the keys above the prefix, then `need` of those matching it (all of them,
+  // but for repeated empty keys)
+  const int total = min(K, m), n_hi = total - need;
+  __syncthreads();
+  if (tid == 0) {
+    s_cnt = 0;
+    s_above = 0;
+  }
+  __syncthreads();
+  for (int e = tid; e < m; e += 256) {
+    const uint64_t k = src.key(i, e0 + e);
+    if ((k & mask) > prefix) {
+      o[atomicAdd(&s_cnt, 1)] = k;
+    } else if ((k & mask) == prefix) {
+      const int p = atomicAdd(&s_above, 1);
+      if (p < need) o[n_hi + p] = k;
+    }
+  }
+  for (int t = total + tid; t < K; t += 256) o[t] = 0;
+}
+
 }  // namespace
 
 cudaError_t launch_merge_bins(const K1Plan& p, Partials parts, float* out_v, int32_t* out_a,
@@ -653,9 +759,6 @@ cudaError_t launch_merge_bins(const K1Plan& p, Partials parts, float* out_v, int
   const unsigned blocks = (unsigned)cdiv(n, 256);
   if (parts.keys64) {
     KeySource s{reinterpret_cast<const uint64_t*>(parts.v), p.L};
-    merge_bins_kernel<<<blocks, 256, 0, st>>>(s, p.M, p.L, out_v, out_a);
-  } else if (parts.a) {
-    PairSource s{parts.v, parts.a, p.M, p.Lk, p.L, p.nsplits, parts.index_offset, p.g};
     merge_bins_kernel<<<blocks, 256, 0, st>>>(s, p.M, p.L, out_v, out_a);
   } else if (parts.merged) {
     MergedSource s{reinterpret_cast<const uint32_t*>(parts.v), p.M, p.Lk, p.L,
@@ -692,10 +795,6 @@ cudaError_t launch_k2(const K1Plan& p, Partials parts, int Kp, const uint64_t* r
     KeySource s{reinterpret_cast<const uint64_t*>(parts.v), p.L};
     return dispatch_k2(s, p, Kp, run_in, out_keys, sorted, st);
   }
-  if (parts.a) {
-    PairSource s{parts.v, parts.a, p.M, p.Lk, p.L, p.nsplits, parts.index_offset, p.g};
-    return dispatch_k2(s, p, Kp, run_in, out_keys, sorted, st);
-  }
   if (parts.merged) {
     MergedSource s{reinterpret_cast<const uint32_t*>(parts.v), p.M, p.Lk, p.L,
                    parts.index_offset, p.g, p.code_bits};
@@ -704,6 +803,39 @@ cudaError_t launch_k2(const K1Plan& p, Partials parts, int Kp, const uint64_t* r
   PackedSource s{reinterpret_cast<const uint32_t*>(parts.v), p.M, p.Lk, p.L, p.nsplits,
                  p.tiles_per_split, parts.index_offset, p.g, p.code_bits};
   return dispatch_k2(s, p, Kp, run_in, out_keys, sorted, st);
+}
+
+int64_t exact_chunk_rows(int K) {
+  // the second launch merges the running K keys and every CTA's in one CTA
+  return std::max<int64_t>(1, kTopkElems / K - 1) * kTopkElems;
+}
+
+size_t exact_cand_bytes(int64_t M, int64_t n, int K) {
+  return (size_t)(M * cdiv(n, kTopkElems) * K) * 8;
+}
+
+cudaError_t launch_exact_topk(const float* scores, int64_t ld, int64_t M, int64_t n, int64_t row0,
+                              int K, const uint64_t* run_in, uint64_t* run_out, uint64_t* cand,
+                              cudaStream_t st) {
+  if (M <= 0 || n <= 0) return cudaSuccess;
+  const int64_t nblk = cdiv(n, kTopkElems);
+  const int64_t nmerge = (run_in ? K : 0) + nblk * K;
+  if (K < 1 || K > kExactMaxK || nmerge > kTopkElems || M * nblk > 0x7fffffffLL)
+    return cudaErrorInvalidValue;
+  const ScoreSource s{scores, ld, row0};
+  if (nblk == 1 && !run_in) {
+    block_topk_kernel<<<(unsigned)M, 256, 0, st>>>(s, n, (int64_t)1, K, run_out);
+    return cudaGetLastError();
+  }
+  block_topk_kernel<<<(unsigned)(M * nblk), 256, 0, st>>>(s, n, nblk, K, cand);
+  const MergeSource ms{run_in, cand, run_in ? K : 0, nblk * K};
+  block_topk_kernel<<<(unsigned)M, 256, 0, st>>>(ms, nmerge, (int64_t)1, K, run_out);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_k2_scores(const float* scores, int64_t ld, int64_t M, int64_t n, int64_t row0,
+                             int K, const uint64_t* run_in, uint64_t* run_out, cudaStream_t st) {
+  return run_k2(ScoreSource{scores, ld, row0}, M, n, K, run_in, run_out, st);
 }
 
 bool k23_supported(int64_t M, int64_t L, int Kp, int K, int D, const float* qf32,

@@ -29,8 +29,8 @@ struct K1Plan {
 };
 
 // Partial results of K1:
-//   pair form   : per (split, query, bin) a float value + int32 index (exact;
-//                 FP32 path);
+//   key form    : per (query, bin) an ordered 64-bit (score, ~row) key merged
+//                 by atomicMax (FP32 and k1_tcs);
 //   packed form : per (split, query, bin) one 32-bit float whose low
 //                 code_bits bits encode the tile ordinal inside the split;
 //   merged form : per (query, bin) the maximum over splits of the packed keys
@@ -38,8 +38,7 @@ struct K1Plan {
 //                 float_to_ordered) so that unsigned atomicMax merges them;
 //                 0 marks a bin no row reached. The array must start at zero.
 struct Partials {
-  float* v;         // pair form values, or packed / merged keys
-  int32_t* a;       // pair form indices (nullptr otherwise)
+  float* v;         // packed / merged keys, 64-bit keys, or plain scores
   int64_t index_offset;  // added to every decoded index (chunked exact search)
   bool merged;
   bool keys64;      // v holds [M][L] 64-bit (score, ~index) keys, 0 = empty
@@ -50,6 +49,10 @@ cudaError_t launch_prep(const float* x, int64_t rows, int D, int pitch, int metr
                         void* out_lp, float* out_scale, float* out_hnorm, float* out_f32,
                         cudaStream_t st, uint32_t* zero_buf = nullptr, int64_t zero_n = 0);
 
+// FP32 K1. Search: the running best of each (query, bin) merges into the
+// [M][L] 64-bit keys (out.keys64; zero on entry). Exact search (out.keys64
+// false): one bin per row (p.L rows), the scores themselves into out.v, rows of
+// round_up(p.L, 4) floats.
 cudaError_t launch_k1_simt(const K1Plan& p, const float* X, const float* hnorm, const float* Qp,
                            Partials out, cudaStream_t st);
 
@@ -61,7 +64,7 @@ cudaError_t launch_k1_tc(const K1Plan& p, const void* X, const float* xscale, co
 // Tensor-core K1 (BF16, rows up to 4096 elements; or E4M3 codes with one
 // database-wide scale xscale[0], IP and COS), queries on TMEM lanes;
 // with bin_map KNN_BINS_MOD each bin's rows sit side by side in the
-// accumulator (the ragged last grid row is scored by a small extra kernel),
+// accumulator,
 // with KNN_BINS_CONTIGUOUS a step is 256 consecutive rows. G[M][L] receives
 // ordered 64-bit (score, ~index) keys by atomicMax and must be zero on entry.
 bool k1_tcs_supported(int dtype, int D, int metric, int64_t N, int64_t L);
@@ -91,6 +94,23 @@ cudaError_t launch_k2(const K1Plan& p, Partials parts, int Kp, const uint64_t* r
 // index (index -1 and value -inf for a bin no row reached).
 cudaError_t launch_merge_bins(const K1Plan& p, Partials parts, float* out_v, int32_t* out_a,
                               cudaStream_t st);
+
+// Top-K of an exact search's chunk: the best K of n scores per query (ld
+// floats apart; -inf and NaN are no candidates; score e is row row0 + e), joined
+// with the K keys per query in run_in (nullptr: none), as a set of K keys per
+// query in run_out. cand: exact_cand_bytes(M, n, K) of scratch.
+// exact_chunk_rows(K): the most rows of a chunk.
+constexpr int kExactMaxK = 1024;
+int64_t exact_chunk_rows(int K);
+size_t exact_cand_bytes(int64_t M, int64_t n, int K);
+cudaError_t launch_exact_topk(const float* scores, int64_t ld, int64_t M, int64_t n, int64_t row0,
+                              int K, const uint64_t* run_in, uint64_t* run_out, uint64_t* cand,
+                              cudaStream_t st);
+
+// The same for K beyond kExactMaxK: one CTA per query streams the scores
+// against the running best K (sorted; run_in and run_out may be one array).
+cudaError_t launch_k2_scores(const float* scores, int64_t ld, int64_t M, int64_t n, int64_t row0,
+                             int K, const uint64_t* run_in, uint64_t* run_out, cudaStream_t st);
 
 // K3: score the Kp candidates of each query in FP32 and keep the best K.
 // Rows come from xf32 (N x D) when given, else from the stored rows.
