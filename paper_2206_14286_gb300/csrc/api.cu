@@ -153,14 +153,18 @@ K1Plan make_plan(int64_t N, int64_t M, int64_t L, int D, int metric, int dtype,
       // SIMT CTAs run two per SM: the split count with the least
       // (waves of 2 * sms CTAs) x (tiles per CTA), the smallest on ties,
       // which also keeps the per-split partials no larger than needed
+      // (for each number of tiles per CTA, the smallest split count with it: the
+      // others only add CTAs)
       const int64_t wave = 2 * sms;
       int64_t best = -1;
-      for (int64_t s = 1; s <= std::min<int64_t>(p.ntiles, 4 * wave); ++s) {
-        const int64_t cost = cdiv(units * s, wave) * cdiv(p.ntiles, s);
+      for (int64_t s = 1; s <= std::min<int64_t>(p.ntiles, 4 * wave);) {
+        const int64_t tiles = cdiv(p.ntiles, s);
+        const int64_t cost = cdiv(units * s, wave) * tiles;
         if (best < 0 || cost < best) {
           best = cost;
           splits = s;
         }
+        s = tiles > 1 ? cdiv(p.ntiles, tiles - 1) : p.ntiles + 1;
       }
     }
     if (dtype != KNN_F32 && sms > 0) {

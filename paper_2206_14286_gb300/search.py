@@ -11,9 +11,24 @@ from ._lib import METRIC, DTYPE, BINS, check
 _ESIZE = {"f32": 4, "bf16": 2, "e4m3": 1, "e4m3t": 1}
 
 
-def _stream(stream):
-    s = stream if stream is not None else torch.cuda.current_stream()
-    return s.cuda_stream
+def _stream(stream, device=None):
+    """Handle of `stream`, or of the current stream of `device` (of the
+    current device if None)."""
+    if stream is not None:
+        return stream.cuda_stream
+    # (torch.cuda.current_stream() builds a Stream object: 3 us)
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device() if device is None
+                                              else device.index)
+
+
+def _call(device, what, fn, *args):
+    """fn(*args) with `device` current, its status checked."""
+    if torch.cuda.current_device() == device.index:
+        rc = fn(*args)
+    else:
+        with torch.cuda.device(device):
+            rc = fn(*args)
+    check(rc, what)
 
 
 def _ptr(t):
@@ -63,12 +78,11 @@ class Database:
             self.f32 = torch.empty((self.N, self.D), dtype=torch.float32, device=dev)
         else:
             self.f32 = x if keep_f32 else None
-        with torch.cuda.device(dev):
-            check(_lib.get().knn_prepare(x.data_ptr(), self.N, self.D, METRIC[metric], DTYPE[dtype],
-                                         self.lp.data_ptr(), _ptr(self.scale), _ptr(self.hnorm),
-                                         _ptr(self.f32) if metric == "cos" else None,
-                                         _stream(stream)), "knn_prepare")
+        _call(dev, "knn_prepare", _lib.get().knn_prepare, x.data_ptr(), self.N, self.D,
+              METRIC[metric], DTYPE[dtype], self.lp.data_ptr(), _ptr(self.scale), _ptr(self.hnorm),
+              _ptr(self.f32) if metric == "cos" else None, _stream(stream, dev))
         self._ws = {}
+        self._plans = {}
 
     # -- helpers ---------------------------------------------------------------
     def _args(self):
@@ -85,6 +99,24 @@ class Database:
     def resolve_L(self, K, L=None, recall_target=0.95):
         return int(L) if L else plan_bins(self.N, K, recall_target)
 
+    def _search_plan(self, M, K, L, recall_target, rerank, bins):
+        """(bins, workspace bytes) of a search with these sizes: a function of
+        the arguments alone, kept for the sizes that come again."""
+        key = (M, K, L, recall_target, rerank, bins)
+        plan = self._plans.get(key)
+        if plan is None:
+            Lr = self.resolve_L(K, L, recall_target)
+            nb = _lib.get().knn_search_workspace(self.N, self.D, DTYPE[self.dtype],
+                                                 METRIC[self.metric], M, K, Lr, BINS[bins],
+                                                 recall_target, rerank)
+            if nb == 0:
+                raise ValueError("invalid search arguments (N=%d D=%d M=%d K=%d L=%d)"
+                                 % (self.N, self.D, M, K, Lr))
+            if len(self._plans) >= 256:
+                self._plans.clear()
+            plan = self._plans[key] = (Lr, nb)
+        return plan
+
     # -- calls -----------------------------------------------------------------
     def search(self, q, K, L=None, recall_target=0.95, rerank=2, stream=None, out=None,
                bins="mod", slot=0):
@@ -95,23 +127,17 @@ class Database:
         streams at the same time use different slots."""
         q = q.contiguous()
         M = q.shape[0]
-        L = self.resolve_L(K, L, recall_target)
         lib = _lib.get()
-        nb = lib.knn_search_workspace(self.N, self.D, DTYPE[self.dtype], METRIC[self.metric], M, K,
-                                      L, BINS[bins], recall_target, rerank)
-        if nb == 0:
-            raise ValueError("invalid search arguments (N=%d D=%d M=%d K=%d L=%d)"
-                             % (self.N, self.D, M, K, L))
+        L, nb = self._search_plan(M, K, L, recall_target, rerank, bins)
         ws = self._get_ws(("search", M, K, L, rerank, bins, slot), nb)
         if out is None:
             val = torch.empty((M, K), dtype=torch.float32, device=self.device)
             idx = torch.empty((M, K), dtype=torch.int32, device=self.device)
         else:
             val, idx = out
-        with torch.cuda.device(self.device):
-            check(lib.knn_search(*self._args(), q.data_ptr(), M, K, L, BINS[bins], recall_target,
-                                 rerank, val.data_ptr(), idx.data_ptr(), ws.data_ptr(),
-                                 ws.numel(), _stream(stream)), "knn_search")
+        _call(self.device, "knn_search", lib.knn_search, *self._args(), q.data_ptr(), M, K, L,
+              BINS[bins], recall_target, rerank, val.data_ptr(), idx.data_ptr(), ws.data_ptr(),
+              ws.numel(), _stream(stream, self.device))
         return val, idx
 
     def search_host(self, q_host, K, L=None, recall_target=0.95, rerank=2, stream=None,
@@ -137,10 +163,10 @@ class Database:
         else:
             val, idx = out
         fn = lib.knn_search_host if wait else lib.knn_search_host_async
-        with torch.cuda.device(self.device):
-            check(fn(*self._args(), q_host.data_ptr(), M, K, L, BINS[bins], recall_target, rerank,
-                     val.data_ptr(), idx.data_ptr(), ws.data_ptr(), ws.numel(), _stream(stream)),
-                  "knn_search_host" if wait else "knn_search_host_async")
+        _call(self.device, "knn_search_host" if wait else "knn_search_host_async", fn,
+              *self._args(), q_host.data_ptr(), M, K, L, BINS[bins], recall_target, rerank,
+              val.data_ptr(), idx.data_ptr(), ws.data_ptr(), ws.numel(),
+              _stream(stream, self.device))
         return val, idx
 
     def search_static(self, q, K, L=None, recall_target=0.95, rerank=2, stream=None, out=None,
@@ -156,11 +182,9 @@ class Database:
             idx = torch.empty((M, K), dtype=torch.int32, device=self.device)
         else:
             val, idx = out
-        with torch.cuda.device(self.device):
-            check(_lib.get().knn_search_static(*self._args(), q.data_ptr(), M, K, L, BINS[bins],
-                                               recall_target, rerank, val.data_ptr(),
-                                               idx.data_ptr(), _stream(stream)),
-                  "knn_search_static")
+        _call(self.device, "knn_search_static", _lib.get().knn_search_static, *self._args(),
+              q.data_ptr(), M, K, L, BINS[bins], recall_target, rerank, val.data_ptr(),
+              idx.data_ptr(), _stream(stream, self.device))
         return val, idx
 
     def search_exact(self, q, K, stream=None):
@@ -174,10 +198,9 @@ class Database:
         ws = self._get_ws(("exact", M, K), nb)
         val = torch.empty((M, K), dtype=torch.float32, device=self.device)
         idx = torch.empty((M, K), dtype=torch.int32, device=self.device)
-        with torch.cuda.device(self.device):
-            check(lib.knn_search_exact(*self._args(), q.data_ptr(), M, K, val.data_ptr(),
-                                       idx.data_ptr(), ws.data_ptr(), ws.numel(),
-                                       _stream(stream)), "knn_search_exact")
+        _call(self.device, "knn_search_exact", lib.knn_search_exact, *self._args(), q.data_ptr(), M,
+              K, val.data_ptr(), idx.data_ptr(), ws.data_ptr(), ws.numel(),
+              _stream(stream, self.device))
         return val, idx
 
     def partial_reduce(self, q, L, stream=None, bins="mod"):
@@ -193,11 +216,9 @@ class Database:
         V = torch.empty((M, L), dtype=torch.float32, device=self.device)
         A = torch.empty((M, L), dtype=torch.int32, device=self.device)
         a = self._args()
-        with torch.cuda.device(self.device):
-            check(lib.knn_partial_reduce(a[0], a[1], a[2], self.N, self.D, a[6], a[7],
-                                         q.data_ptr(), M, L, BINS[bins], V.data_ptr(),
-                                         A.data_ptr(), ws.data_ptr(), ws.numel(),
-                                         _stream(stream)), "knn_partial_reduce")
+        _call(self.device, "knn_partial_reduce", lib.knn_partial_reduce, a[0], a[1], a[2], self.N,
+              self.D, a[6], a[7], q.data_ptr(), M, L, BINS[bins], V.data_ptr(), A.data_ptr(),
+              ws.data_ptr(), ws.numel(), _stream(stream, self.device))
         return V, A
 
     def backward(self, q, idx, grad_val, want_dq=True, want_dx=True, deterministic=False,
@@ -230,13 +251,11 @@ class Database:
             raise ValueError("atomic=True is the non-deterministic mode")
         nb = lib.knn_backward_workspace(self.N, self.D, M, K, int(deterministic))
         ws = self._get_ws(("bwd", M, K), nb) if (nb and want_dx and not atomic) else None
-        with torch.cuda.device(self.device):
-            check(lib.knn_backward(self.lp.data_ptr(), _ptr(self.scale), _ptr(xf), self.N, self.D,
-                                   DTYPE[self.dtype], METRIC[self.metric], q.data_ptr(), M, K,
-                                   idx.data_ptr(), grad_val.data_ptr(), _ptr(dq), _ptr(dx),
-                                   int(bool(zero_dx)), int(deterministic), _ptr(ws),
-                                   ws.numel() if ws is not None else 0, _stream(stream)),
-                  "knn_backward")
+        _call(self.device, "knn_backward", lib.knn_backward, self.lp.data_ptr(), _ptr(self.scale),
+              _ptr(xf), self.N, self.D, DTYPE[self.dtype], METRIC[self.metric], q.data_ptr(), M, K,
+              idx.data_ptr(), grad_val.data_ptr(), _ptr(dq), _ptr(dx), int(bool(zero_dx)),
+              int(deterministic), _ptr(ws), ws.numel() if ws is not None else 0,
+              _stream(stream, self.device))
         return dq, dx
 
 
@@ -252,10 +271,9 @@ class OwnedDatabase:
         self.N, self.D = x.shape
         self.metric, self.dtype, self.device = metric, dtype, x.device
         h = ctypes.c_void_p()
-        with torch.cuda.device(x.device):
-            check(_lib.get().knn_db_create(x.data_ptr(), self.N, self.D, METRIC[metric],
-                                           DTYPE[dtype], int(bool(keep_f32)), _stream(stream),
-                                           ctypes.byref(h)), "knn_db_create")
+        _call(x.device, "knn_db_create", _lib.get().knn_db_create, x.data_ptr(), self.N, self.D,
+              METRIC[metric], DTYPE[dtype], int(bool(keep_f32)), _stream(stream, x.device),
+              ctypes.byref(h))
         self.handle = h
         self._ws = None
 
@@ -271,16 +289,14 @@ class OwnedDatabase:
             self._ws = _workspace(nb, self.device)
         val = torch.empty((M, K), dtype=torch.float32, device=self.device)
         idx = torch.empty((M, K), dtype=torch.int32, device=self.device)
-        with torch.cuda.device(self.device):
-            check(lib.knn_db_search(self.handle, q.data_ptr(), M, K, L, BINS[bins], recall_target,
-                                    rerank, val.data_ptr(), idx.data_ptr(), self._ws.data_ptr(),
-                                    self._ws.numel(), _stream(stream)), "knn_db_search")
+        _call(self.device, "knn_db_search", lib.knn_db_search, self.handle, q.data_ptr(), M, K, L,
+              BINS[bins], recall_target, rerank, val.data_ptr(), idx.data_ptr(),
+              self._ws.data_ptr(), self._ws.numel(), _stream(stream, self.device))
         return val, idx
 
     def close(self):
         if self.handle is not None and self.handle.value:
-            with torch.cuda.device(self.device):
-                check(_lib.get().knn_db_destroy(self.handle), "knn_db_destroy")
+            _call(self.device, "knn_db_destroy", _lib.get().knn_db_destroy, self.handle)
         self.handle = None
 
 
@@ -307,12 +323,10 @@ def approx_max_k(scores, K, L=None, recall_target=0.95, bins="mod", is_min=False
     val = torch.empty((M, width), dtype=torch.float32, device=S.device)
     idx = torch.empty((M, width), dtype=torch.int32, device=S.device)
     ws = _workspace(nb, S.device)
-    with torch.cuda.device(S.device):
-        check(lib.knn_approx_max_k(S.data_ptr(), dt, M, N, int(K), Lr, int(planning_size),
-                                   recall_target, BINS[bins], int(bool(is_min)),
-                                   int(bool(aggregate_to_topk)), val.data_ptr(), idx.data_ptr(),
-                                   ws.data_ptr(), ws.numel(), _stream(stream)),
-              "knn_approx_max_k")
+    _call(S.device, "knn_approx_max_k", lib.knn_approx_max_k, S.data_ptr(), dt, M, N, int(K), Lr,
+          int(planning_size), recall_target, BINS[bins], int(bool(is_min)),
+          int(bool(aggregate_to_topk)), val.data_ptr(), idx.data_ptr(), ws.data_ptr(), ws.numel(),
+          _stream(stream, S.device))
     return val, idx
 
 
