@@ -411,10 +411,16 @@ knn_status search_impl(const SearchArgs& a, float* out_val, int32_t* out_idx, vo
                    a.metric, qf32, q_stride, a.db_f32, a.N, out_val, out_idx, st);
     return cuda_status(e);
   }
+  if (rescore_supported(s.plan, s.Kp)) {
+    ProfScope ps(2, st);
+    e = launch_rescore(s.plan, parts, s.Kp, a.K, qf32, q_stride, a.db_f32, a.db_lp,
+                       stored_dtype(a.dtype), a.db_scale, a.N, out_val, out_idx, st);
+    return cuda_status(e);
+  }
   uint64_t* cand = reinterpret_cast<uint64_t*>(ws + s.off_cand);
   {
     ProfScope ps(2, st);
-    e = launch_k2(s.plan, parts, s.Kp, nullptr, cand, st, /*sorted=*/false);
+    e = launch_k2(s.plan, parts, s.Kp, cand, st, /*sorted=*/false);
   }
   if (e != cudaSuccess) return cuda_status(e);
   {
@@ -851,19 +857,9 @@ knn_status knn_approx_max_k(const void* scores, int32_t score_dtype, int64_t M, 
   if (!aggregate_to_topk)
     return cuda_status(launch_keys_to_pairs(reinterpret_cast<const uint64_t*>(G), M * Lr,
                                             is_min ? 1 : 0, out_val, out_idx, st));
-  K1Plan p{};
-  p.M = M;
-  p.N = N;
-  p.L = Lr;
-  p.Lk = Lr;
-  p.g = 1;
-  p.nsplits = 1;
-  Partials parts{reinterpret_cast<float*>(G), 0, false, true};
   uint64_t* keys = reinterpret_cast<uint64_t*>(ws + al((size_t)M * Lr * 8));
-  e = launch_k2(p, parts, K, nullptr, keys, st);
-  if (e == cudaSuccess)
-    e = launch_keys_to_pairs(keys, M * K, is_min ? 1 : 0, out_val, out_idx, st);
-  return cuda_status(e);
+  return cuda_status(launch_k2_pairs(reinterpret_cast<const uint64_t*>(G), M, Lr, K, is_min ? 1 : 0,
+                                     keys, out_val, out_idx, st));
 }
 
 size_t knn_search_exact_workspace(int64_t N, int32_t D, int32_t dtype, int32_t metric, int64_t M,
@@ -1025,7 +1021,9 @@ knn_status knn_shard_rescore(const int64_t* keys, int64_t M, int64_t L, int32_t 
   p.g = 1;
   p.nsplits = 1;
   Partials parts{reinterpret_cast<float*>(G), 0, false, true};
-  if (e == cudaSuccess) e = launch_k2(p, parts, Kp, nullptr, cand, st, /*sorted=*/false);
+  // sorted: the shards' candidate arrays merge element by element, so every
+  // shard has to hold the candidates in the same order
+  if (e == cudaSuccess) e = launch_k2(p, parts, Kp, cand, st, /*sorted=*/true);
   const float* qf = q;
   int64_t q_stride = D;
   if (e == cudaSuccess && metric == KNN_COS) {
@@ -1064,17 +1062,9 @@ knn_status knn_shard_finish(const int64_t* cand_keys, int64_t M, int32_t Kp, int
   uint64_t* C = reinterpret_cast<uint64_t*>(ws);
   uint64_t* top = reinterpret_cast<uint64_t*>(ws + al((size_t)M * Kp * 8));
   cudaError_t e = launch_signed_to_keys(cand_keys, M * Kp, C, st);
-  K1Plan p{};
-  p.M = M;
-  p.L = Kp;
-  p.Lk = Kp;
-  p.g = 1;
-  p.nsplits = 1;
-  Partials parts{reinterpret_cast<float*>(C), 0, false, true};
-  if (e == cudaSuccess) e = launch_k2(p, parts, K, nullptr, top, st);
   // internal scores are larger-is-better: L2 reports the squared distance
   if (e == cudaSuccess)
-    e = launch_keys_to_pairs(top, M * K, metric == KNN_L2 ? 1 : 0, out_val, out_idx, st);
+    e = launch_k2_pairs(C, M, Kp, K, metric == KNN_L2 ? 1 : 0, top, out_val, out_idx, st);
   return cuda_status(e);
 }
 

@@ -1,17 +1,16 @@
 // k2_topk.cu -- ExactRescoring (Sec. 5): per query, merge the partial bin
 // winners of every split (and fold) and select the best Kp (score, index)
-// pairs, sorted best first.
+// keys; fused with the FP32 re-rank for searches (rescore_kernel, k23_kernel).
 //
-// One CTA per query. Candidates stream through shared memory against a
-// threshold (the current Kp-th best key): only keys above it are appended to
-// a buffer, and when the buffer could overflow it is sorted together with
-// the running best Kp (bitonic, descending) and truncated. With the L bin
-// winners of one query this is a single bitonic sort of O(L log^2 L) work, the
-// paper's ExactRescoring; the same code streams the N scores of a chunked
-// exact search.
+// One CTA per query holds its L <= 8192 keys in registers. Up to Kp = 128 the
+// Kp-th largest of the 256 threads' maxima bounds the selection from below:
+// few keys beyond Kp reach it, and those are gathered and sorted. Larger Kp: a
+// radix select. More candidates (L > 8192, or Kp > 1024) stream through
+// shared memory against the running Kp-th best key.
 #include <algorithm>
 
 #include "common.cuh"
+#include "dtypes.cuh"
 #include "kernels.h"
 
 namespace tpuknn {
@@ -103,60 +102,6 @@ __device__ __forceinline__ uint64_t shfl_xor_u64(uint64_t v, int o) {
   return ((uint64_t)hi << 32) | lo;
 }
 
-// Lane `lane`'s candidates b = lane + 32 r (r < KPL) of query i, 0 past L.
-template <class Src, int KPL>
-__device__ __forceinline__ void lane_keys(const Src& src, int64_t i, int lane, int64_t L,
-                                          uint64_t (&k)[KPL]) {
-#pragma unroll
-  for (int r = 0; r < KPL; ++r) {
-    const int64_t b = lane + 32 * r;
-    k[r] = b < L ? src.key(i, b) : 0;
-  }
-}
-// One warp per query: lane l holds candidates l, l+32, ... (KPL of them),
-// sorted; Kp rounds each take the warp-wide maximum of the lane heads and pop
-// it from its lane. Keys are unique (distinct indices), so one lane pops.
-template <class Src, int KPL>
-__global__ void __launch_bounds__(256)
-k2_warp_kernel(Src src, int64_t M, int64_t L, int Kp, uint64_t* __restrict__ out_keys) {
-  const int lane = threadIdx.x & 31;
-  const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (i >= M) return;
-  uint64_t k[KPL];
-  lane_keys(src, i, lane, L, k);
-  reg_sort_desc<KPL>(k);
-  for (int r = 0; r < Kp; ++r) {
-    uint64_t m = k[0];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      const uint64_t y = shfl_xor_u64(m, o);
-      m = y > m ? y : m;
-    }
-    if (lane == 0) out_keys[i * Kp + r] = m;
-    if (m != 0 && k[0] == m) {
-#pragma unroll
-      for (int t = 0; t + 1 < KPL; ++t) k[t] = k[t + 1];
-      k[KPL - 1] = 0;
-    }
-  }
-}
-
-template <class Src>
-cudaError_t run_k2_warp(const Src& src, int64_t M, int64_t L, int Kp, uint64_t* out,
-                        cudaStream_t st) {
-  const int kpl = next_pow2((int)cdiv(L, 32));
-  const unsigned blocks = (unsigned)cdiv(M * 32, 256);
-  switch (kpl) {
-    case 1: k2_warp_kernel<Src, 1><<<blocks, 256, 0, st>>>(src, M, L, Kp, out); break;
-    case 2: k2_warp_kernel<Src, 2><<<blocks, 256, 0, st>>>(src, M, L, Kp, out); break;
-    case 4: k2_warp_kernel<Src, 4><<<blocks, 256, 0, st>>>(src, M, L, Kp, out); break;
-    case 8: k2_warp_kernel<Src, 8><<<blocks, 256, 0, st>>>(src, M, L, Kp, out); break;
-    case 16: k2_warp_kernel<Src, 16><<<blocks, 256, 0, st>>>(src, M, L, Kp, out); break;
-    default: k2_warp_kernel<Src, 32><<<blocks, 256, 0, st>>>(src, M, L, Kp, out); break;
-  }
-  return cudaGetLastError();
-}
-
 template <class Src>
 __global__ void __launch_bounds__(256)
 k2_topk_kernel(Src src, int64_t nelem, int Kp, int CH, int CAP, const uint64_t* __restrict__ run_in,
@@ -232,7 +177,7 @@ cudaError_t run_k2(const Src& src, int64_t M, int64_t nelem, int Kp, const uint6
 }
 
 // ExactRescoring and the FP32 re-rank in one CTA of 4 warps per query, for
-// the merged 64-bit keys of K1 (L <= 1024, Kp <= 32, K <= 32, 16-byte
+// the merged 64-bit keys of K1 (L <= 256, Kp <= 32, K <= 32, 16-byte
 // aligned FP32 rows with D % 4 == 0). Warp 0 takes the best Kp of the L keys:
 // each lane sorts its KPL keys, then every round the warp's maximum key
 // comes from two 32-bit max-reductions (high word, then the low word among
@@ -252,7 +197,7 @@ k23_kernel(const uint64_t* __restrict__ G, int64_t L, int Kp, int K, int D,
   __shared__ uint64_t s_key[32];
   const int64_t i = blockIdx.x;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  pdl_wait();  // the keys come from the contraction (and the ragged-row kernel)
+  pdl_wait();  // the keys come from the contraction
   pdl_trigger();  // the next call's query prep may launch (it waits for this kernel)
   if (warp == 0) {
     uint64_t k[KPL];
@@ -364,96 +309,11 @@ cudaError_t run_k23(const uint64_t* G, int64_t M, int64_t L, int Kp, int K, int 
     K23_CASE(2)
     K23_CASE(4)
     K23_CASE(8)
-    K23_CASE(16)
-    K23_CASE(32)
     default: return cudaErrorNotSupported;
   }
 #undef K23_CASE
 }
 
-
-// Up to 2048 candidates and 256 selected per query (no running input): a CTA
-// of 8 warps per query. Warp w sorts candidates [256 w, 256 w + 256) held in
-// registers, element e = 32 r + lane in register r, by a bitonic network
-// (partners within a lane swap registers, partners across lanes exchange by
-// shuffle). Three merge rounds then halve the sorted lists: the top 256 of two
-// descending lists A and B are max(A[e], B[255 - e]), a bitonic sequence that
-// eight more bitonic steps sort. The result is the best Kp keys in order, as
-// from the CTA kernel, at O(L log^2 256) compare-exchanges instead of full
-// sorts of the whole buffer.
-__device__ __forceinline__ void wsort_step(uint64_t (&k)[8], int lane, int size, int stride,
-                                           bool all_desc) {
-  if (stride >= 32) {
-    const int rs = stride >> 5;
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      if ((r & rs) == 0) {
-        const int e = r * 32 + lane;
-        const bool desc = all_desc || (e & size) == 0;
-        const uint64_t a = k[r], b = k[r | rs];
-        const bool sw = desc ? (a < b) : (a > b);
-        k[r] = sw ? b : a;
-        k[r | rs] = sw ? a : b;
-      }
-    }
-  } else {
-#pragma unroll
-    for (int r = 0; r < 8; ++r) {
-      const int e = r * 32 + lane;
-      const bool desc = all_desc || (e & size) == 0;
-      const uint64_t o = shfl_xor_u64(k[r], stride);
-      const bool lower = (lane & stride) == 0;
-      const bool keep_max = (lower == desc);
-      k[r] = keep_max ? (o > k[r] ? o : k[r]) : (o < k[r] ? o : k[r]);
-    }
-  }
-}
-
-template <class Src>
-__global__ void __launch_bounds__(256)
-k2_wsort_kernel(Src src, int64_t L, int Kp, uint64_t* __restrict__ out_keys) {
-  __shared__ uint64_t lists[8][256];
-  const int64_t i = blockIdx.x;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  uint64_t k[8];
-#pragma unroll
-  for (int r = 0; r < 8; ++r) {
-    const int64_t b = (int64_t)warp * 256 + r * 32 + lane;
-    k[r] = b < L ? src.key(i, b) : 0;
-  }
-#pragma unroll
-  for (int size = 2; size <= 256; size <<= 1)
-#pragma unroll
-    for (int stride = size >> 1; stride > 0; stride >>= 1) wsort_step(k, lane, size, stride, false);
-#pragma unroll
-  for (int r = 0; r < 8; ++r) lists[warp][r * 32 + lane] = k[r];
-  for (int level = 1; level < 8; level <<= 1) {
-    __syncthreads();
-    if ((warp & (2 * level - 1)) == 0) {
-      const uint64_t* B = lists[warp + level];
-#pragma unroll
-      for (int r = 0; r < 8; ++r) {
-        const int e = r * 32 + lane;
-        const uint64_t a = lists[warp][e], b = B[255 - e];
-        k[r] = a > b ? a : b;
-      }
-#pragma unroll
-      for (int stride = 128; stride > 0; stride >>= 1) wsort_step(k, lane, 256, stride, true);
-      __syncwarp();
-#pragma unroll
-      for (int r = 0; r < 8; ++r) lists[warp][r * 32 + lane] = k[r];
-    }
-  }
-  __syncthreads();
-  for (int t = threadIdx.x; t < Kp; t += blockDim.x) out_keys[i * Kp + t] = lists[0][t];
-}
-
-template <class Src>
-cudaError_t run_k2_wsort(const Src& src, int64_t M, int64_t L, int Kp, uint64_t* out,
-                         cudaStream_t st) {
-  k2_wsort_kernel<Src><<<(unsigned)M, 256, 0, st>>>(src, L, Kp, out);
-  return cudaGetLastError();
-}
 
 // Warp 0 of a radix-select pass: the digit where the count of the histogram's
 // bins from the top reaches `need`, the keys in the bins above it, and
@@ -505,80 +365,334 @@ __device__ __forceinline__ void pick_digit(const uint32_t* hist, int need, int l
   }
 }
 
-// The best Kp of a query's L keys as a set, in no particular order (for the
-// re-rank, which orders its candidates itself): one CTA of 256 threads per
-// query holds the L keys in registers (KPT per thread, L <= 256 KPT) and
-// finds the Kp-th largest key T by a radix select over the 64 key bits, 8 per
-// pass from the most significant: per pass a 256-bin histogram in shared
-// memory of the keys that match the digits chosen so far, and warp 0 picks
-// the digit where the count from the top reaches Kp. It stops once every key
-// matching the chosen digits is needed. Output: the keys above the chosen
-// digits, then as many matching keys as still needed (all of them but for
-// repeated empty keys, 0). Keys are distinct otherwise, so this is the set
-// of the Kp largest, the same set a sort would keep.
-template <class Src, int KPT>
-__global__ void __launch_bounds__(256)
-k2_select_kernel(Src src, int64_t L, int Kp, uint64_t* __restrict__ out_keys) {
-  __shared__ uint32_t hist[256];
-  __shared__ int s_digit, s_above, s_stop, s_hi, s_eq;
-  const int64_t i = blockIdx.x;
-  const int tid = threadIdx.x, lane = tid & 31;
-  uint64_t k[KPT];
+constexpr int kTopkElems = 8192, kTopkCap = 1024, kThrMaxK = 128;
+
+// The selection of one CTA of 256 threads.
+struct SelectSmem {
+  uint64_t buf[kTopkCap];
+  uint32_t w[256];  // maxima, or a histogram
+  int cnt, digit, above, stop;
+};
+
+// The K-th largest of the 256 threads' x (K <= 256): a bitonic sort, one value
+// per thread.
+__device__ __forceinline__ uint32_t kth_of_threads(uint32_t x, int K, uint32_t* w) {
+  const int tid = threadIdx.x;
 #pragma unroll
-  for (int u = 0; u < KPT; ++u) {
-    const int64_t b = (int64_t)u * 256 + tid;
-    k[u] = b < L ? src.key(i, b) : 0;
+  for (int size = 2; size <= 256; size <<= 1) {
+#pragma unroll
+    for (int stride = size >> 1; stride > 0; stride >>= 1) {
+      uint32_t y;
+      if (stride >= 32) {
+        __syncthreads();
+        w[tid] = x;
+        __syncthreads();
+        y = w[tid ^ stride];
+      } else {
+        y = __shfl_xor_sync(0xffffffffu, x, stride);
+      }
+      const bool keep_max = ((tid & stride) == 0) == ((tid & size) == 0);
+      x = keep_max ? max(x, y) : min(x, y);
+    }
+  }
+  __syncthreads();
+  w[tid] = x;
+  __syncthreads();
+  return w[K - 1];
+}
+
+// The keys of buf[0..c), c <= kTopkCap, sorted best first; buf is zero from c
+// to `fill` afterwards. All 256 threads; ends with a barrier.
+__device__ __forceinline__ void sort_buf(uint64_t* buf, int c, int fill) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (c <= 32) {
+    if (tid < 32) {
+      uint64_t x = lane < c ? buf[lane] : 0;
+#pragma unroll
+      for (int size = 2; size <= 32; size <<= 1) {
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+          const uint64_t y = shfl_xor_u64(x, stride);
+          const bool keep_max = ((lane & stride) == 0) == ((lane & size) == 0);
+          x = keep_max ? (y > x ? y : x) : (y < x ? y : x);
+        }
+      }
+      buf[lane] = x;
+    }
+    for (int t = 32 + tid; t < fill; t += 256) buf[t] = 0;
+    __syncthreads();
+    return;
+  }
+  const int P2 = next_pow2(c);
+  for (int t = c + tid; t < max(P2, fill); t += 256) buf[t] = 0;
+  bitonic_sort_desc(buf, P2);
+}
+
+// The best Kp <= kTopkCap of the CTA's L keys (thread t holds keys t + 256 u)
+// into sm.buf[0..Kp): sorted best first if `sorted`, else as a set.
+//
+// Up to kThrMaxK: the Kp-th largest of the threads' maxima (high words) is a
+// lower bound of the Kp-th largest key; the keys that reach it are gathered.
+// Beyond, or if more reach it than the buffer holds (ties): a radix select,
+// 8 bits per pass from the top, a 256-bin histogram of the keys that match
+// the digits chosen so far, stopping once every matching key is needed. Keys
+// are distinct but for empty ones (0), so the set is that of a sort.
+template <int KPT>
+__device__ __forceinline__ void select_topk(const uint64_t (&k)[KPT], int L, int Kp, bool sorted,
+                                            SelectSmem& sm) {
+  const int tid = threadIdx.x, lane = tid & 31;
+  bool radix = Kp > kThrMaxK;
+  if (tid == 0) sm.cnt = 0;
+  if (!radix) {
+    uint32_t mx = 0;
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) mx = max(mx, (uint32_t)(k[u] >> 32));
+    const uint32_t thr = max(kth_of_threads(mx, Kp, sm.w), 1u);
+#pragma unroll
+    for (int u = 0; u < KPT; ++u) {
+      if ((uint32_t)(k[u] >> 32) >= thr) {
+        const int p = atomicAdd(&sm.cnt, 1);
+        if (p < kTopkCap) sm.buf[p] = k[u];
+      }
+    }
+    __syncthreads();
+    const int c = sm.cnt;
+    radix = c > kTopkCap;
+    if (!radix) {
+      if (sorted || c > Kp) {
+        sort_buf(sm.buf, c, Kp);
+      } else {
+        for (int t = c + tid; t < Kp; t += 256) sm.buf[t] = 0;
+        __syncthreads();
+      }
+      return;
+    }
   }
   uint64_t prefix = 0, mask = 0;
-  int need = Kp;  // keys still to take among those matching the prefix
+  int need = min(Kp, L);  // keys still to take among those matching the prefix
   for (int shift = 56; shift >= 0; shift -= 8) {
-    hist[tid] = 0;
+    __syncthreads();
+    sm.w[tid] = 0;
     __syncthreads();
 #pragma unroll
     for (int u = 0; u < KPT; ++u)
-      if ((int64_t)u * 256 + tid < L && (k[u] & mask) == prefix)
-        atomicAdd(&hist[(uint32_t)(k[u] >> shift) & 255u], 1u);
+      if (u * 256 + tid < L && (k[u] & mask) == prefix)
+        atomicAdd(&sm.w[(uint32_t)(k[u] >> shift) & 255u], 1u);
     __syncthreads();
-    if (tid < 32) pick_digit(hist, need, lane, s_digit, s_above, s_stop);
+    if (tid < 32) pick_digit(sm.w, need, lane, sm.digit, sm.above, sm.stop);
     __syncthreads();
-    prefix |= (uint64_t)s_digit << shift;
+    prefix |= (uint64_t)sm.digit << shift;
     mask |= (uint64_t)0xFF << shift;
-    need -= s_above;
-    const bool stop = s_stop != 0;
-    __syncthreads();  // s_* are rewritten by the next pass
-    if (stop) break;
+    need -= sm.above;
+    if (sm.stop) break;
   }
   // the keys above the prefix (masked), then `need` of those matching it
+  const int n_hi = min(Kp, L) - need;
+  __syncthreads();
   if (tid == 0) {
-    s_hi = 0;
-    s_eq = 0;
+    sm.cnt = 0;
+    sm.above = 0;
   }
   __syncthreads();
-  uint64_t* out = out_keys + i * Kp;
-  const int n_hi = Kp - need;
 #pragma unroll
   for (int u = 0; u < KPT; ++u) {
-    if ((int64_t)u * 256 + tid >= L) continue;
+    if (u * 256 + tid >= L) continue;
     const uint64_t m = k[u] & mask;
     if (m > prefix) {
-      out[atomicAdd(&s_hi, 1)] = k[u];
+      sm.buf[atomicAdd(&sm.cnt, 1)] = k[u];
     } else if (m == prefix) {
-      const int p = atomicAdd(&s_eq, 1);
-      if (p < need) out[n_hi + p] = k[u];
+      const int p = atomicAdd(&sm.above, 1);
+      if (p < need) sm.buf[n_hi + p] = k[u];
+    }
+  }
+  for (int t = L + tid; t < Kp; t += 256) sm.buf[t] = 0;  // Kp > L: empty
+  __syncthreads();
+  if (sorted) sort_buf(sm.buf, Kp, Kp);
+}
+
+template <class Src, int KPT>
+__device__ __forceinline__ void load_keys(const Src& src, int64_t i, int L, uint64_t (&k)[KPT]) {
+#pragma unroll
+  for (int u = 0; u < KPT; ++u) {
+    const int b = u * 256 + threadIdx.x;
+    k[u] = b < L ? src.key(i, b) : 0;
+  }
+}
+
+// ExactRescoring alone: the best Kp keys of each query, as keys or (out_val
+// given) as values, negated when `neg`, and indices.
+// (three CTAs per SM with up to 8192 keys: 10,000 queries 1.18 -> 0.86 ms)
+template <class Src, int KPT>
+__global__ void __launch_bounds__(256, KPT == 32 ? 3 : 4)
+k2_select_kernel(Src src, int L, int Kp, bool sorted, uint64_t* __restrict__ out_keys, int neg,
+                 float* __restrict__ out_val, int32_t* __restrict__ out_idx) {
+  __shared__ SelectSmem sm;
+  const int64_t i = blockIdx.x;
+  pdl_wait();
+  uint64_t k[KPT];
+  load_keys(src, i, L, k);
+  select_topk(k, L, Kp, sorted, sm);
+  for (int t = threadIdx.x; t < Kp; t += 256) {
+    const uint64_t key = sm.buf[t];
+    if (out_val) {
+      out_val[i * Kp + t] =
+          key ? (neg ? -key_score(key) : key_score(key)) : __int_as_float(0x7fc00000);
+      out_idx[i * Kp + t] = key ? key_index(key) : -1;
+    } else {
+      out_keys[i * Kp + t] = key;
     }
   }
 }
 
+// ExactRescoring and the FP32 re-rank of its Kp candidates in one launch: the
+// candidates stay in shared memory, the 8 warps score four of them at a time
+// (eight in the re-rank alone; their row loads in flight together), and the
+// best K of the exact keys are sorted and written: 4096 queries, L = 605, 64
+// candidates of 256 elements 160 -> 75 us, against one warp per query for the
+// selection and a second launch. The re-rank alone of 2000 x 800 rows of 96:
+// 224 -> 180 us (3.4 TB/s of gathered rows). The scores are those of the separate re-rank, sum by
+// sum: VEC4 (Kp <= 32, 16-byte aligned FP32 rows) a lane owns 4 adjacent
+// elements of each 128, else every 32nd element. KPT = 0: the re-rank alone, of
+// Kp <= 1024 candidates that src holds.
+struct RescoreArgs {
+  int L, Kp, K, D, metric, dtype, pitch;
+  const float* qf32;
+  int64_t q_stride;
+  const float* xf32;
+  const void* xlp;
+  const float* xscale;
+  int64_t N;
+  float* out_val;
+  int32_t* out_idx;
+};
+
+template <class Src, int KPT, bool VEC4>
+__global__ void __launch_bounds__(256) rescore_kernel(Src src, RescoreArgs a) {
+  __shared__ SelectSmem sm;
+  const int64_t i = blockIdx.x;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  pdl_wait();     // the keys come from the contraction
+  pdl_trigger();  // the next call's query prep may launch (it waits for this kernel)
+  if constexpr (KPT == 0) {
+    for (int t = tid; t < a.Kp; t += 256) sm.buf[t] = src.key(i, t);
+    __syncthreads();
+  } else {
+    uint64_t k[KPT];
+    load_keys(src, i, a.L, k);
+    select_topk(k, a.L, a.Kp, false, sm);
+  }
+  const float* q = a.qf32 + i * a.q_stride;
+  constexpr int kCand = KPT == 0 ? 8 : 4;
+  for (int c0 = warp * kCand; c0 < a.Kp; c0 += 8 * kCand) {
+    int32_t jj[kCand];
+    float acc[kCand];
+#pragma unroll
+    for (int u = 0; u < kCand; ++u) {
+      const uint64_t key = c0 + u < a.Kp ? sm.buf[c0 + u] : 0;
+      const int32_t j = key ? key_index(key) : -1;
+      jj[u] = (j >= 0 && j < a.N) ? j : -1;
+      acc[u] = 0.0f;
+    }
+    if constexpr (VEC4) {
+      for (int d0 = 0; d0 < a.D; d0 += 128) {
+        const int d = d0 + lane * 4;
+        const bool in = d < a.D;
+        const float4 qv = in ? *reinterpret_cast<const float4*>(q + d) : make_float4(0, 0, 0, 0);
+        float4 xv[kCand];
+#pragma unroll
+        for (int u = 0; u < kCand; ++u)
+          xv[u] = (in && jj[u] >= 0)
+                      ? __ldg(reinterpret_cast<const float4*>(a.xf32 + (int64_t)jj[u] * a.D + d))
+                      : make_float4(0, 0, 0, 0);
+#pragma unroll
+        for (int u = 0; u < kCand; ++u) {
+          if (a.metric == KNN_L2) {
+            // elements past D contribute 0: both sides are zero there
+            const float t0 = qv.x - xv[u].x, t1 = qv.y - xv[u].y, t2 = qv.z - xv[u].z,
+                        t3 = qv.w - xv[u].w;
+            acc[u] = fmaf(t0, t0, acc[u]);
+            acc[u] = fmaf(t1, t1, acc[u]);
+            acc[u] = fmaf(t2, t2, acc[u]);
+            acc[u] = fmaf(t3, t3, acc[u]);
+          } else {
+            acc[u] = fmaf(qv.x, xv[u].x, acc[u]);
+            acc[u] = fmaf(qv.y, xv[u].y, acc[u]);
+            acc[u] = fmaf(qv.z, xv[u].z, acc[u]);
+            acc[u] = fmaf(qv.w, xv[u].w, acc[u]);
+          }
+        }
+      }
+    } else {
+      for (int d = lane; d < a.D; d += 32) {
+        const float qq = q[d];
+        float xv[kCand];
+#pragma unroll
+        for (int u = 0; u < kCand; ++u)
+          xv[u] = jj[u] < 0 ? 0.0f
+                            : (a.xf32 ? a.xf32[(int64_t)jj[u] * a.D + d]
+                                      : load_stored(a.xlp, a.dtype, jj[u], a.pitch, d, a.xscale));
+#pragma unroll
+        for (int u = 0; u < kCand; ++u) {
+          if (a.metric == KNN_L2) {
+            const float t = qq - xv[u];
+            acc[u] = fmaf(t, t, acc[u]);
+          } else {
+            acc[u] = fmaf(qq, xv[u], acc[u]);
+          }
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kCand; ++u) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc[u] += __shfl_xor_sync(0xffffffffu, acc[u], o);
+    }
+    __syncwarp();  // every lane has read these candidates
+    if (lane == 0) {
+#pragma unroll
+      for (int u = 0; u < kCand; ++u)
+        if (c0 + u < a.Kp)
+          sm.buf[c0 + u] =
+              jj[u] < 0 ? 0 : make_key(a.metric == KNN_L2 ? -acc[u] : acc[u], jj[u]);
+    }
+  }
+  __syncthreads();
+  if (a.Kp <= 256 || a.K > kThrMaxK) {
+    sort_buf(sm.buf, a.Kp, a.Kp);
+  } else {
+    // many candidates, few wanted: select again, from registers
+    uint64_t k[kTopkCap / 256];
+#pragma unroll
+    for (int u = 0; u < kTopkCap / 256; ++u) {
+      const int c = u * 256 + tid;
+      k[u] = c < a.Kp ? sm.buf[c] : 0;
+    }
+    __syncthreads();
+    select_topk(k, a.Kp, a.K, true, sm);
+  }
+  for (int t = tid; t < a.K; t += 256) {
+    const uint64_t key = sm.buf[t];
+    const float sc = key_score(key);
+    a.out_idx[i * a.K + t] = key ? key_index(key) : -1;
+    a.out_val[i * a.K + t] =
+        key ? (a.metric == KNN_L2 ? -sc : sc) : __int_as_float(0x7fc00000);
+  }
+}
+
 template <class Src>
-cudaError_t run_k2_select(const Src& src, int64_t M, int64_t L, int Kp, uint64_t* out,
-                          cudaStream_t st) {
-  if (L <= 2048)
-    k2_select_kernel<Src, 8><<<(unsigned)M, 256, 0, st>>>(src, L, Kp, out);
-  else if (L <= 4096)
-    k2_select_kernel<Src, 16><<<(unsigned)M, 256, 0, st>>>(src, L, Kp, out);
-  else
-    k2_select_kernel<Src, 32><<<(unsigned)M, 256, 0, st>>>(src, L, Kp, out);
-  return cudaGetLastError();
+cudaError_t run_k2_select(const Src& src, int64_t M, int64_t L, int Kp, bool sorted, uint64_t* out,
+                          int neg, float* out_val, int32_t* out_idx, cudaStream_t st) {
+  auto kern = L <= 1024   ? k2_select_kernel<Src, 4>
+              : L <= 2048 ? k2_select_kernel<Src, 8>
+              : L <= 4096 ? k2_select_kernel<Src, 16>
+                          : k2_select_kernel<Src, 32>;
+  return launch_pdl(kern, dim3((unsigned)M), dim3(256), 0, st, src, (int)L, Kp, sorted, out, neg,
+                    out_val, out_idx);
+}
+template <class Src, bool VEC4>
+cudaError_t run_rescore(const Src& src, int64_t M, const RescoreArgs& a, cudaStream_t st) {
+  auto kern = a.L <= 1024 ? rescore_kernel<Src, 4, VEC4> : rescore_kernel<Src, 8, VEC4>;
+  return launch_pdl(kern, dim3((unsigned)M), dim3(256), 0, st, src, a);
 }
 
 // ---------------------------------------------------------------------------
@@ -595,8 +709,6 @@ cudaError_t run_k2_select(const Src& src, int64_t M, int64_t L, int Kp, uint64_t
 // or more elements at the bound than the buffer holds (ties): a radix select
 // over the keys, read again in every pass.
 // ---------------------------------------------------------------------------
-constexpr int kTopkElems = 8192, kTopkCap = 1024, kThrMaxK = 128;
-
 // Scores of a chunk: element e of query i as an ordered 64-bit key (0: no
 // candidate, which -inf and NaN are not). raw() is what a thread loads, with
 // no condition around it, so that its loads are all in flight together.
@@ -633,15 +745,13 @@ template <class Src>
 __global__ void __launch_bounds__(256)
 block_topk_kernel(Src src, int64_t n, int64_t nblk, int K, uint64_t* __restrict__ out) {
   constexpr int KPT = kTopkElems / 256;
-  __shared__ uint64_t buf[kTopkCap];
-  __shared__ uint32_t s_mx[256];
-  __shared__ int s_cnt, s_digit, s_above, s_stop;
+  __shared__ SelectSmem sm;
   const int tid = threadIdx.x, lane = tid & 31;
   const int64_t i = blockIdx.x / nblk, blk = blockIdx.x % nblk;
   const int64_t e0 = blk * kTopkElems;
   const int m = (int)min((int64_t)kTopkElems, n - e0);  // elements of this CTA
   uint64_t* o = out + (i * nblk + blk) * K;
-  if (tid == 0) s_cnt = 0;
+  if (tid == 0) sm.cnt = 0;
   bool overflow = K > kThrMaxK;
   if (!overflow) {
     typename Src::Raw raw[KPT];
@@ -653,97 +763,56 @@ block_topk_kernel(Src src, int64_t n, int64_t nblk, int K, uint64_t* __restrict_
       h[u] = u * 256 + tid < m ? Src::high(raw[u]) : 0u;
       mx = max(mx, h[u]);
     }
-    // descending sort of the 256 maxima: bitonic, one per thread
-    uint32_t x = mx;
-#pragma unroll
-    for (int size = 2; size <= 256; size <<= 1) {
-#pragma unroll
-      for (int stride = size >> 1; stride > 0; stride >>= 1) {
-        uint32_t y;
-        if (stride >= 32) {
-          __syncthreads();
-          s_mx[tid] = x;
-          __syncthreads();
-          y = s_mx[tid ^ stride];
-        } else {
-          y = __shfl_xor_sync(0xffffffffu, x, stride);
-        }
-        const bool keep_max = ((tid & stride) == 0) == ((tid & size) == 0);
-        x = keep_max ? max(x, y) : min(x, y);
-      }
-    }
-    __syncthreads();
-    s_mx[tid] = x;
-    __syncthreads();
-    const uint32_t thr = max(s_mx[K - 1], 1u);
+    const uint32_t thr = max(kth_of_threads(mx, K, sm.w), 1u);
 #pragma unroll
     for (int u = 0; u < KPT; ++u) {
       if (h[u] >= thr) {
-        const int p = atomicAdd(&s_cnt, 1);
-        if (p < kTopkCap) buf[p] = src.key(i, e0 + u * 256 + tid);
+        const int p = atomicAdd(&sm.cnt, 1);
+        if (p < kTopkCap) sm.buf[p] = src.key(i, e0 + u * 256 + tid);
       }
     }
     __syncthreads();
-    overflow = s_cnt > kTopkCap;
+    overflow = sm.cnt > kTopkCap;
   }
   if (!overflow) {
-    const int c = s_cnt;
-    if (c <= 32) {
-      if (tid >= 32) return;
-      uint64_t x = lane < c ? buf[lane] : 0;
-#pragma unroll
-      for (int size = 2; size <= 32; size <<= 1) {
-#pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
-          const uint64_t y = shfl_xor_u64(x, stride);
-          const bool keep_max = ((lane & stride) == 0) == ((lane & size) == 0);
-          x = keep_max ? (y > x ? y : x) : (y < x ? y : x);
-        }
-      }
-      for (int t = lane; t < K; t += 32) o[t] = t < 32 ? x : 0;
-      return;
-    }
-    const int P2 = next_pow2(c);
-    for (int t = c + tid; t < P2; t += 256) buf[t] = 0;
-    bitonic_sort_desc(buf, P2);
-    for (int t = tid; t < K; t += 256) o[t] = t < P2 ? buf[t] : 0;
+    sort_buf(sm.buf, sm.cnt, K);
+    for (int t = tid; t < K; t += 256) o[t] = sm.buf[t];
     return;
   }
   // radix select, 8 bits per pass from the top, over the keys in memory
-  uint32_t* hist = s_mx;
   uint64_t prefix = 0, mask = 0;
   int need = min(K, m);
   for (int shift = 56; shift >= 0; shift -= 8) {
     __syncthreads();
-    hist[tid] = 0;
+    sm.w[tid] = 0;
     __syncthreads();
     for (int e = tid; e < m; e += 256) {
       const uint64_t k = src.key(i, e0 + e);
-      if ((k & mask) == prefix) atomicAdd(&hist[(uint32_t)(k >> shift) & 255u], 1u);
+      if ((k & mask) == prefix) atomicAdd(&sm.w[(uint32_t)(k >> shift) & 255u], 1u);
     }
     __syncthreads();
-    if (tid < 32) pick_digit(hist, need, lane, s_digit, s_above, s_stop);
+    if (tid < 32) pick_digit(sm.w, need, lane, sm.digit, sm.above, sm.stop);
     __syncthreads();
-    prefix |= (uint64_t)s_digit << shift;
+    prefix |= (uint64_t)sm.digit << shift;
     mask |= (uint64_t)0xFF << shift;
-    need -= s_above;
-    if (s_stop) break;
+    need -= sm.above;
+    if (sm.stop) break;
   }
   // the keys above the prefix, then `need` of those matching it (all of them,
   // but for repeated empty keys)
   const int total = min(K, m), n_hi = total - need;
   __syncthreads();
   if (tid == 0) {
-    s_cnt = 0;
-    s_above = 0;
+    sm.cnt = 0;
+    sm.above = 0;
   }
   __syncthreads();
   for (int e = tid; e < m; e += 256) {
     const uint64_t k = src.key(i, e0 + e);
     if ((k & mask) > prefix) {
-      o[atomicAdd(&s_cnt, 1)] = k;
+      o[atomicAdd(&sm.cnt, 1)] = k;
     } else if ((k & mask) == prefix) {
-      const int p = atomicAdd(&s_above, 1);
+      const int p = atomicAdd(&sm.above, 1);
       if (p < need) o[n_hi + p] = k;
     }
   }
@@ -752,57 +821,91 @@ block_topk_kernel(Src src, int64_t n, int64_t nblk, int K, uint64_t* __restrict_
 
 }  // namespace
 
+// Per query: one CTA with the candidates in registers up to 8192 of them and
+// 1024 selected; the streaming CTA kernel everything else.
+template <class Src>
+cudaError_t dispatch_k2(const Src& s, const K1Plan& p, int Kp, uint64_t* out_keys, bool sorted,
+                        cudaStream_t st) {
+  if (p.L <= kTopkElems && Kp <= kTopkCap && p.M <= 0x7fffffffLL)
+    return run_k2_select(s, p.M, p.L, Kp, sorted, out_keys, 0, nullptr, nullptr, st);
+  return run_k2(s, p.M, p.L, Kp, nullptr, out_keys, st);
+}
+
+// f(source) for the form the partials have.
+template <class F>
+cudaError_t with_source(const K1Plan& p, const Partials& parts, F f) {
+  if (parts.keys64) return f(KeySource{reinterpret_cast<const uint64_t*>(parts.v), p.L});
+  if (parts.merged)
+    return f(MergedSource{reinterpret_cast<const uint32_t*>(parts.v), p.M, p.Lk, p.L,
+                          parts.index_offset, p.g, p.code_bits});
+  return f(PackedSource{reinterpret_cast<const uint32_t*>(parts.v), p.M, p.Lk, p.L, p.nsplits,
+                        p.tiles_per_split, parts.index_offset, p.g, p.code_bits});
+}
+
 cudaError_t launch_merge_bins(const K1Plan& p, Partials parts, float* out_v, int32_t* out_a,
                               cudaStream_t st) {
   const int64_t n = p.M * p.L;
   if (n <= 0) return cudaSuccess;
-  const unsigned blocks = (unsigned)cdiv(n, 256);
-  if (parts.keys64) {
-    KeySource s{reinterpret_cast<const uint64_t*>(parts.v), p.L};
-    merge_bins_kernel<<<blocks, 256, 0, st>>>(s, p.M, p.L, out_v, out_a);
-  } else if (parts.merged) {
-    MergedSource s{reinterpret_cast<const uint32_t*>(parts.v), p.M, p.Lk, p.L,
-                   parts.index_offset, p.g, p.code_bits};
-    merge_bins_kernel<<<blocks, 256, 0, st>>>(s, p.M, p.L, out_v, out_a);
-  } else {
-    PackedSource s{reinterpret_cast<const uint32_t*>(parts.v), p.M, p.Lk, p.L, p.nsplits,
-                   p.tiles_per_split, parts.index_offset, p.g, p.code_bits};
-    merge_bins_kernel<<<blocks, 256, 0, st>>>(s, p.M, p.L, out_v, out_a);
-  }
-  return cudaGetLastError();
+  return with_source(p, parts, [&](auto s) {
+    merge_bins_kernel<<<(unsigned)cdiv(n, 256), 256, 0, st>>>(s, p.M, p.L, out_v, out_a);
+    return cudaGetLastError();
+  });
 }
 
-// Per query: the warp kernel serves up to 1024 candidates and 64 selected,
-// the sorting CTA kernel up to 2048 candidates and 256 selected (both with
-// no running input); beyond those, when an unordered set will do, the radix
-// select up to 8192 candidates; the streaming CTA kernel everything else.
-template <class Src>
-cudaError_t dispatch_k2(const Src& s, const K1Plan& p, int Kp, const uint64_t* run_in,
-                        uint64_t* out_keys, bool sorted, cudaStream_t st) {
-  if (run_in == nullptr && p.L <= 1024 && Kp <= 64) return run_k2_warp(s, p.M, p.L, Kp, out_keys, st);
-  if (run_in == nullptr && p.L <= 2048 && Kp <= 256 && p.M <= 0x7fffffffLL)
-    return run_k2_wsort(s, p.M, p.L, Kp, out_keys, st);
-  // a set is enough (the re-rank orders it): radix select instead of sorts
-  if (!sorted && run_in == nullptr && p.L <= 8192 && p.M <= 0x7fffffffLL)
-    return run_k2_select(s, p.M, p.L, Kp, out_keys, st);
-  return run_k2(s, p.M, p.L, Kp, run_in, out_keys, st);
-}
-
-cudaError_t launch_k2(const K1Plan& p, Partials parts, int Kp, const uint64_t* run_in,
-                      uint64_t* out_keys, cudaStream_t st, bool sorted) {
+cudaError_t launch_k2(const K1Plan& p, Partials parts, int Kp, uint64_t* out_keys, cudaStream_t st,
+                      bool sorted) {
   if (p.M <= 0) return cudaSuccess;
-  if (parts.keys64) {
-    KeySource s{reinterpret_cast<const uint64_t*>(parts.v), p.L};
-    return dispatch_k2(s, p, Kp, run_in, out_keys, sorted, st);
-  }
-  if (parts.merged) {
-    MergedSource s{reinterpret_cast<const uint32_t*>(parts.v), p.M, p.Lk, p.L,
-                   parts.index_offset, p.g, p.code_bits};
-    return dispatch_k2(s, p, Kp, run_in, out_keys, sorted, st);
-  }
-  PackedSource s{reinterpret_cast<const uint32_t*>(parts.v), p.M, p.Lk, p.L, p.nsplits,
-                 p.tiles_per_split, parts.index_offset, p.g, p.code_bits};
-  return dispatch_k2(s, p, Kp, run_in, out_keys, sorted, st);
+  return with_source(
+      p, parts, [&](auto s) { return dispatch_k2(s, p, Kp, out_keys, sorted, st); });
+}
+
+cudaError_t launch_k2_pairs(const uint64_t* keys, int64_t M, int64_t L, int K, int neg,
+                            uint64_t* scratch, float* out_val, int32_t* out_idx,
+                            cudaStream_t st) {
+  if (M <= 0) return cudaSuccess;
+  const KeySource s{keys, L};
+  if (L <= kTopkElems && K <= kTopkCap && M <= 0x7fffffffLL)
+    return run_k2_select(s, M, L, K, true, nullptr, neg, out_val, out_idx, st);
+  cudaError_t e = run_k2(s, M, L, K, nullptr, scratch, st);
+  return e == cudaSuccess ? launch_keys_to_pairs(scratch, M * K, neg, out_val, out_idx, st) : e;
+}
+
+// (With up to 8192 keys the selection holds 64 registers of them a thread and
+// two CTAs fit an SM, too few for the re-rank's row loads: 2M x 96 E4M3 rows, L
+// = 8192, 800 candidates, 2000 queries, 1.107 ms a search against 1.011 with
+// two launches.)
+bool rescore_supported(const K1Plan& p, int Kp) {
+  return p.L <= 2048 && Kp <= kTopkCap && p.M <= 0x7fffffffLL;
+}
+
+cudaError_t launch_rescore(const K1Plan& p, Partials parts, int Kp, int K, const float* qf32,
+                           int64_t q_stride, const float* xf32, const void* xlp, int dtype,
+                           const float* xscale, int64_t N, float* out_val, int32_t* out_idx,
+                           cudaStream_t st) {
+  if (p.M <= 0) return cudaSuccess;
+  if (!rescore_supported(p, Kp)) return cudaErrorNotSupported;
+  const RescoreArgs a{(int)p.L, Kp,   K,   p.D,    p.metric, dtype,   p.pitch, qf32,
+                      q_stride, xf32, xlp, xscale, N,        out_val, out_idx};
+  // the sums of the separate re-rank's vector kernel, where that would run
+  const bool vec4 = Kp <= 32 && K <= 32 && xf32 && p.D % 4 == 0 && q_stride % 4 == 0 &&
+                    (reinterpret_cast<uintptr_t>(xf32) & 15) == 0 &&
+                    (reinterpret_cast<uintptr_t>(qf32) & 15) == 0;
+  return with_source(p, parts, [&](auto s) {
+    return vec4 ? run_rescore<decltype(s), true>(s, p.M, a, st)
+                : run_rescore<decltype(s), false>(s, p.M, a, st);
+  });
+}
+
+cudaError_t launch_rerank(int64_t M, int D, int metric, const uint64_t* cand, int Kp, int K,
+                          const float* qf32, int64_t q_stride, const float* xf32, const void* xlp,
+                          int dtype, int pitch, const float* xscale, int64_t N, float* out_val,
+                          int32_t* out_idx, cudaStream_t st) {
+  if (M <= 0) return cudaSuccess;
+  if (Kp > kTopkCap || M > 0x7fffffffLL) return cudaErrorNotSupported;
+  const RescoreArgs a{Kp,       Kp,   K,   D,      metric, dtype,   pitch, qf32,
+                      q_stride, xf32, xlp, xscale, N,      out_val, out_idx};
+  return launch_pdl(rescore_kernel<KeySource, 0, false>, dim3((unsigned)M), dim3(256), 0, st,
+                    KeySource{cand, Kp}, a);
 }
 
 int64_t exact_chunk_rows(int K) {
@@ -840,7 +943,7 @@ cudaError_t launch_k2_scores(const float* scores, int64_t ld, int64_t M, int64_t
 
 bool k23_supported(int64_t M, int64_t L, int Kp, int K, int D, const float* qf32,
                    int64_t q_stride, const float* xf32) {
-  return M > 0 && M <= 0x7fffffffLL && L >= 1 && L <= 1024 && Kp >= 1 && Kp <= 32 &&
+  return M > 0 && M <= 0x7fffffffLL && L >= 1 && L <= 256 && Kp >= 1 && Kp <= 32 &&
          K >= 1 && K <= 32 && xf32 && D % 4 == 0 && q_stride % 4 == 0 &&
          (reinterpret_cast<uintptr_t>(xf32) & 15) == 0 &&
          (reinterpret_cast<uintptr_t>(qf32) & 15) == 0;

@@ -3,7 +3,8 @@
 // the candidates, FP32 decides their order and values).
 //
 // Kp <= 32: one warp per query (k3_warp4_kernel for 16-byte aligned FP32
-// rows, k3_warp_kernel otherwise), the keys sorted across the lanes. Larger
+// rows, k3_warp_kernel otherwise), the keys sorted across the lanes. Up to
+// 1024: launch_rerank. Larger
 // Kp: one CTA per query; each warp scores four candidates at a time with lanes
 // splitting D (coalesced row reads), then the Kp keys are sorted in shared
 // memory. Values: IP <q,x>; L2 sum (q-x)^2 evaluated directly; COS <q,x> of
@@ -252,6 +253,9 @@ cudaError_t launch_k3(int64_t M, int D, int metric, const uint64_t* cand, int Kp
         out_idx);
     return cudaGetLastError();
   }
+  if (Kp <= 1024)
+    return launch_rerank(M, D, metric, cand, Kp, K, qf32, q_stride, xf32, xlp, dtype, pitch, xscale,
+                         N, out_val, out_idx, st);
   const int P2 = next_pow2(Kp > K ? Kp : K);
   const size_t smem = (size_t)P2 * sizeof(uint64_t);
   if (smem > 200 * 1024) return cudaErrorInvalidValue;

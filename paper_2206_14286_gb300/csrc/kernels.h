@@ -83,12 +83,29 @@ cudaError_t launch_keys_to_pairs(const uint64_t* keys, int64_t n, int neg, float
                                  int32_t* out_a, cudaStream_t st);
 
 // K2: per query, merge the partials of every split and fold and select the
-// best Kp (score, index) keys, sorted. If run_in is given its Kp keys per
-// query join the selection (running top-K of a chunked search). With
-// sorted = false the keys may come in any order (for the re-rank, which
-// orders its candidates itself).
-cudaError_t launch_k2(const K1Plan& p, Partials parts, int Kp, const uint64_t* run_in,
-                      uint64_t* out_keys, cudaStream_t st, bool sorted = true);
+// best Kp (score, index) keys, sorted best first; with sorted = false in any
+// order (for a re-rank, which orders its candidates itself).
+cudaError_t launch_k2(const K1Plan& p, Partials parts, int Kp, uint64_t* out_keys, cudaStream_t st,
+                      bool sorted = true);
+
+// The best K of M x L keys as values (negated when neg) and indices, best
+// first; scratch: M x K keys.
+cudaError_t launch_k2_pairs(const uint64_t* keys, int64_t M, int64_t L, int K, int neg,
+                            uint64_t* scratch, float* out_val, int32_t* out_idx, cudaStream_t st);
+
+// K2 and K3 in one launch (L <= 2048, Kp <= 1024): the same results as
+// launch_k2 followed by launch_k3.
+bool rescore_supported(const K1Plan& p, int Kp);
+cudaError_t launch_rescore(const K1Plan& p, Partials parts, int Kp, int K, const float* qf32,
+                           int64_t q_stride, const float* xf32, const void* xlp, int dtype,
+                           const float* xscale, int64_t N, float* out_val, int32_t* out_idx,
+                           cudaStream_t st);
+
+// The re-rank of 32 < Kp <= 1024 candidates (launch_k3's kernel for them).
+cudaError_t launch_rerank(int64_t M, int D, int metric, const uint64_t* cand, int Kp, int K,
+                          const float* qf32, int64_t q_stride, const float* xf32, const void* xlp,
+                          int dtype, int pitch, const float* xscale, int64_t N, float* out_val,
+                          int32_t* out_idx, cudaStream_t st);
 
 // PartialReduce output alone: per (query, bin) the merged best value and
 // index (index -1 and value -inf for a bin no row reached).
@@ -116,7 +133,8 @@ cudaError_t launch_k2_scores(const float* scores, int64_t ld, int64_t M, int64_t
 // Rows come from xf32 (N x D) when given, else from the stored rows.
 // ExactRescoring and the FP32 re-rank fused (one CTA of 4 warps per query)
 // for K1's merged [M][L] keys; the same results as launch_k2 followed by
-// launch_k3. Supported when k23_supported(...) holds (L <= 1024, Kp <= 32,
+// launch_k3, by four warps per query, for few bins. Supported when
+// k23_supported(...) holds (L <= 256, Kp <= 32,
 // K <= 32, 16-byte aligned FP32 rows and queries with D % 4 == 0);
 // otherwise returns cudaErrorNotSupported.
 bool k23_supported(int64_t M, int64_t L, int Kp, int K, int D, const float* qf32,

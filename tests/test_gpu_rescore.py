@@ -1,0 +1,59 @@
+"""ExactRescoring, alone (approx_max_k's sorted top-K) and fused with the FP32
+re-rank (search), on small integers: scores are exact and mostly tie, so values
+and indices are decided, at the edges of the kernels' candidate and K limits."""
+import pytest
+import torch
+
+from paper_2206_14286_gb300 import search as S
+from tests.gpu_util import ensure_built
+
+pytestmark = pytest.mark.gpu
+
+
+def ints(shape, seed, lo, hi):
+    g = torch.Generator(device="cuda")
+    g.manual_seed(seed)
+    return torch.randint(lo, hi, shape, generator=g, device="cuda").float()
+
+
+def ranked(s, K):
+    o = torch.sort(s, dim=1, descending=True, stable=True)
+    return o.values[:, :K], o.indices[:, :K]
+
+
+@pytest.mark.parametrize("L", [1, 31, 33, 255, 256, 257, 1024, 1025, 2048, 2049, 4096, 4097, 8192,
+                               8193])
+def test_sorted_selection(L):
+    ensure_built()
+    M = 9
+    for hi in (2, 50, 1 << 20):           # nearly all equal, many ties, few ties
+        s = ints((M, L), L + hi, 0, hi)
+        for K in {1, 32, 33, 127, 128, 129, 1000, 1024, 1025, L}:
+            if K > min(L, 4096):
+                continue
+            v, i = S.approx_max_k(s, K, L=L)
+            rv, ri = ranked(s, K)
+            assert torch.equal(v, rv)
+            assert torch.equal(i.long(), ri)
+
+
+@pytest.mark.parametrize("metric", ["ip", "l2"])
+@pytest.mark.parametrize("N", [40, 256, 257, 1000, 1024, 2000, 2048, 2049, 4097, 8192, 8193])
+def test_rescored_search(metric, N):
+    """Every row its own bin and a re-rank of r K: the exact top-K, through
+    rows of 16-byte multiples and not."""
+    ensure_built()
+    for D in (24, 27):
+        x, q = ints((N, D), N + D, -2, 3), ints((37, D), D, -2, 3)
+        d = S.Database(x, metric=metric, dtype="f32")
+        s = q @ x.t()
+        if metric == "l2":
+            s = -((q * q).sum(1)[:, None] + (x * x).sum(1)[None, :] - 2.0 * s)
+        for K, r in ((1, 1), (10, 1), (10, 2), (16, 2), (17, 2), (33, 1), (40, 8), (64, 2), (100, 8),
+                     (129, 2), (200, 6), (500, 4)):
+            if K > N:
+                continue
+            val, idx = d.search(q, K, L=N, rerank=r)
+            rv, ri = ranked(s, K)
+            assert torch.equal(idx.long(), ri)
+            assert torch.equal(val, -rv if metric == "l2" else rv)

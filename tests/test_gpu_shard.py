@@ -99,3 +99,23 @@ def test_sharded_search_equals_the_whole_database(dtype, metric, shards):
     wv, wi = host(wv), host(wi)
     same = np.mean([len(set(gi[k]) & set(wi[k])) / K for k in range(M)])
     assert same > (0.99 if dtype != "e4m3" else 0.97), same
+
+
+@pytest.mark.parametrize("K,rr", [(10, 2), (64, 2), (100, 4), (200, 5)])
+def test_shards_hold_their_candidates_in_the_same_order(K, rr):
+    """The candidate arrays merge element by element: with few or many
+    candidates, the sharded answer is that of the whole database (small
+    integers: every score exact)."""
+    ensure_built()
+    g = np.random.Generator(np.random.PCG64(K))
+    N, D, M, L, shards = 20011, 32, 40, 1024, 3
+    X = g.integers(-3, 4, (N, D)).astype(np.float32)
+    Q = g.integers(-3, 4, (M, D)).astype(np.float32)
+    q = dev(Q)
+    parts = [SH.DatabaseShard(dev(X[r0:r0 + n]), r0, N, "ip", "f32")
+             for r0, n in SH.shard_bounds(N, shards, L)]
+    keys = torch.stack([p.partial(q, L) for p in parts]).amax(0)
+    cand = torch.stack([p.rescore(keys, q, K, rr, L) for p in parts]).amax(0)
+    val, idx = parts[0].finish(cand, K)
+    wv, wi = db(X, "ip", "f32").search(q, K, L=L, rerank=rr)
+    assert torch.equal(idx, wi) and torch.equal(val, wv)
