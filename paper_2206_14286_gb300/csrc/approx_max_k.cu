@@ -28,104 +28,126 @@ __device__ __forceinline__ float load_score(const void* S, int64_t t, float sg) 
   return sg * v + 0.0f;
 }
 
-// Bins j mod L: thread b of a row owns bin b and walks its columns b, b + L,
-// ... of a chunk of kchunk grid rows; neighbouring threads read neighbouring
-// columns, so every pass over a grid row is one coalesced sweep.
-template <int DT>
+// Bins j mod L: a thread owns V bins b0 .. b0 + V - 1 of a row and walks their
+// columns, every bdy-th grid row of the CTA's chunk of grid rows, keeping each
+// bin's best value and grid row in registers (strict '>' while the column
+// grows keeps the smaller column on ties). V = 8 BF16 or 4 FP32 columns of one
+// 16-byte load (L and N multiples of V, S 16-byte aligned), else V = 1.
+//
+// Bound by HBM. threadIdx.x runs over the vectors of a grid row, however many
+// there are (tpr of them, up to 256), and threadIdx.y over grid rows, so the
+// CTA's threads read bdy whole grid rows, which are adjacent in memory, and no
+// lane idles for padding: rounded up to warps, 22 vectors of L = 176 left 10 of
+// 32 lanes without work (1024 x 1M BF16: 510 us). The bdy rows' bests merge in
+// shared memory before one atomicMax per bin.
+template <int DT, int V>
 __global__ void __launch_bounds__(256)
-bin_max_mod_kernel(const void* __restrict__ S, int64_t N, int64_t L, int64_t kchunk, int neg,
+bin_max_mod_kernel(const void* __restrict__ S, int64_t N, int L, int kchunk, int neg,
                    unsigned long long* __restrict__ G) {
-  const int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  constexpr int kEsz = DT == KNN_BF16 ? 2 : 4, U = V == 1 ? 8 : 4;
+  __shared__ uint64_t part[V == 1 ? 1 : V][256];
+  const int tid = threadIdx.y * blockDim.x + threadIdx.x, bdy = blockDim.y;
   const int64_t i = blockIdx.y;
-  if (b >= L) return;
-  const int64_t k0 = (int64_t)blockIdx.z * kchunk;
-  const int64_t k1 = min(cdiv(N, L), k0 + kchunk);
+  const int b0 = ((int)blockIdx.x * blockDim.x + threadIdx.x) * V;
+  const bool live = b0 < L;
+  const uint32_t T = (uint32_t)((N + L - 1) / L);  // grid rows, the last one maybe ragged
+  const uint32_t k0 = blockIdx.z * (uint32_t)kchunk, k1 = min(T, k0 + kchunk);
   const float sg = neg ? -1.0f : 1.0f;
-  uint64_t best = 0;
-  // eight independent loads in flight per thread
-  for (int64_t k = k0; k < k1; k += 8) {
-    float v[8];
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int64_t j = (k + u) * L + b;
-      v[u] = (k + u < k1 && j < N) ? load_score<DT>(S, i * N + j, sg) : 0.0f;
-    }
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      const int64_t j = (k + u) * L + b;
-      if (k + u < k1 && j < N) {
-        const uint64_t key = make_key(v[u], (int32_t)j);
-        best = key > best ? key : best;
-      }
-    }
-  }
-  if (best) atomicMax(&G[i * L + b], (unsigned long long)best);
-}
-
-// The same with 16-byte loads (L and N multiples of the V columns a load holds,
-// S 16-byte aligned): thread (x, y) of a CTA owns bins V*t .. V*t + V - 1,
-// t = blockIdx.x * blockDim.x + x, of row blockIdx.y * blockDim.y + y, and
-// keeps each bin's best value and column (strict '>' in increasing column
-// order keeps the smaller column on ties; the keys made at the end merge
-// across CTAs by atomicMax). A warp reads 32 consecutive 16-byte pieces of a
-// grid row, and each thread has four loads in flight.
-template <int DT>
-__global__ void __launch_bounds__(256)
-bin_max_mod_vec_kernel(const void* __restrict__ S, int64_t M, int64_t N, int64_t L,
-                       int64_t kchunk, int neg, unsigned long long* __restrict__ G) {
-  constexpr int V = DT == KNN_BF16 ? 8 : 4;  // columns per 16-byte load
-  constexpr int kEsz = DT == KNN_BF16 ? 2 : 4;
-  const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const int64_t i = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
-  if (t * V >= L || i >= M) return;
-  const int64_t k0 = (int64_t)blockIdx.z * kchunk;
-  const int64_t k1 = min(cdiv(N, L), k0 + kchunk);
-  const float sg = neg ? -1.0f : 1.0f;
-  const char* row = static_cast<const char*>(S) + i * N * kEsz;
   float bv[V];
-  int32_t bj[V];
+  uint32_t bk[V], bo = 0;  // V = 1: the best score in the keys' order (NaN above all)
+  constexpr uint32_t kNone = 0xffffffffu;
 #pragma unroll
   for (int c = 0; c < V; ++c) {
     bv[c] = neg_inf();
-    bj[c] = -1;
+    bk[c] = kNone;
   }
-  for (int64_t k = k0; k < k1; k += 4) {
-    uint4 raw[4];
+  if (live) {
+    const char* row = static_cast<const char*>(S) + (i * N + b0) * kEsz;
+    // every grid row but the last is whole
+    const uint32_t kfull = (int64_t)(k1 - 1) * L + b0 + V <= N ? k1 : k1 - 1;
+    auto take = [&](const uint4& raw, float one, uint32_t k) {
+      float x[V];
+      if constexpr (V == 1) {
+        x[0] = one;
+      } else if constexpr (DT == KNN_BF16) {
+        const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&raw);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int64_t j0 = (k + u) * L + t * V;
-      raw[u] = (k + u < k1 && j0 < N)
-                   ? __ldg(reinterpret_cast<const uint4*>(row + j0 * kEsz))
-                   : make_uint4(0, 0, 0, 0);
-    }
+        for (int c = 0; c < V; ++c) x[c] = __bfloat162float(h[c]);
+      } else {
+        const float* f = reinterpret_cast<const float*>(&raw);
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
-      const int64_t j0 = (k + u) * L + t * V;
-      if (k + u < k1 && j0 < N) {
-        float x[V];
-        if constexpr (DT == KNN_BF16) {
-          const __nv_bfloat16* h = reinterpret_cast<const __nv_bfloat16*>(&raw[u]);
+        for (int c = 0; c < V; ++c) x[c] = f[c];
+      }
 #pragma unroll
-          for (int c = 0; c < V; ++c) x[c] = __bfloat162float(h[c]);
-        } else {
-          const float* f = reinterpret_cast<const float*>(&raw[u]);
-#pragma unroll
-          for (int c = 0; c < V; ++c) x[c] = f[c];
-        }
-#pragma unroll
-        for (int c = 0; c < V; ++c) {
-          const float v = sg * x[c] + 0.0f;
-          if (bj[c] < 0 || v > bv[c]) {
-            bv[c] = v;
-            bj[c] = (int32_t)(j0 + c);
+      for (int c = 0; c < V; ++c) {
+        // adding +0 turns -0 into +0: the two zeros tie
+        const float v = sg * x[c] + 0.0f;
+        if constexpr (V == 1) {
+          const uint32_t o = float_to_ordered(v);
+          if (o > bo) {
+            bo = o;
+            bk[c] = k;
           }
+        } else if (bk[c] == kNone || v > bv[c]) {
+          bv[c] = v;
+          bk[c] = k;
         }
       }
+    };
+    auto load = [&](uint32_t k, uint4& raw, float& one) {
+      const char* p = row + (int64_t)k * L * kEsz;
+      if constexpr (V == 1)
+        one = load_score<DT>(p, 0, 1.0f);
+      else
+        raw = __ldg(reinterpret_cast<const uint4*>(p));
+    };
+    uint32_t k = k0 + threadIdx.y;
+    for (; k + (U - 1) * bdy < kfull; k += U * bdy) {
+      uint4 raw[U];
+      float one[U];
+#pragma unroll
+      for (int u = 0; u < U; ++u) load(k + u * bdy, raw[u], one[u]);
+#pragma unroll
+      for (int u = 0; u < U; ++u) take(raw[u], one[u], k + u * bdy);
+    }
+    for (; k < kfull; k += bdy) {
+      uint4 raw;
+      float one;
+      load(k, raw, one);
+      take(raw, one, k);
     }
   }
+  auto key = [&](int c) -> uint64_t {
+    if (bk[c] == kNone) return (uint64_t)0;
+    const int32_t j = (int32_t)(bk[c] * (uint32_t)L + b0 + c);
+    return V == 1 ? ((uint64_t)bo << 32) | (uint32_t)~j : make_key(bv[c], j);
+  };
+  if (bdy == 1) {
 #pragma unroll
-  for (int c = 0; c < V; ++c)
-    if (bj[c] >= 0) atomicMax(&G[i * L + t * V + c], (unsigned long long)make_key(bv[c], bj[c]));
+    for (int c = 0; c < V; ++c) {
+      const uint64_t best = key(c);
+      if (best) atomicMax(&G[i * L + b0 + c], (unsigned long long)best);
+    }
+    return;
+  }
+#pragma unroll
+  for (int c = 0; c < V; ++c) {
+    if constexpr (V == 1)
+      part[0][tid] = key(c);
+    else
+      part[c][tid] = key(c);
+  }
+  __syncthreads();
+  for (int t = tid; t < (int)blockDim.x * V; t += blockDim.x * bdy) {
+    const int c = t / blockDim.x, x = t % blockDim.x;
+    const int b = ((int)blockIdx.x * blockDim.x + x) * V + c;
+    uint64_t best = 0;
+    for (int y = 0; y < bdy; ++y) {
+      const uint64_t o = part[c][y * blockDim.x + x];
+      best = o > best ? o : best;
+    }
+    if (best && b < L) atomicMax(&G[i * L + b], (unsigned long long)best);
+  }
 }
 
 __device__ __forceinline__ int64_t runs_bin_of(int64_t j, int64_t q, int64_t r) {
@@ -268,42 +290,27 @@ cudaError_t launch_bin_max(const void* S, int dtype, int64_t M, int64_t N, int64
   }
   const int sms = device_sm_count();
   const int vcols = dtype == KNN_BF16 ? 8 : 4;
-  if (bin_map == KNN_BINS_MOD && L % vcols == 0 && N % vcols == 0 &&
-      (reinterpret_cast<uintptr_t>(S) & 15) == 0) {
-    // 16-byte loads: a CTA is rows x threads, the threads of a row covering
-    // its L / vcols vectors of a grid row
-    const int64_t tpr = L / vcols;
-    const int bdx = (int)std::min<int64_t>(256, round_up(tpr, 32));
-    const int bdy = 256 / bdx;
-    const int64_t bx = cdiv(tpr, bdx), by = cdiv(M, bdy);
+  if (bin_map == KNN_BINS_MOD) {
+    const bool vec = L % vcols == 0 && N % vcols == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0;
+    const int64_t tpr = vec ? L / vcols : L;  // threads that cover a grid row
     const int64_t grid_rows = cdiv(N, L);
-    int64_t kz = cdiv((int64_t)sms * 8, bx * by);
-    if (kz > grid_rows) kz = grid_rows;
-    if (kz < 1) kz = 1;
-    if (kz > 65535) kz = 65535;
+    const int bdx = (int)std::min<int64_t>(256, tpr);
+    const int bdy = (int)std::max<int64_t>(1, std::min<int64_t>(256 / bdx, grid_rows));
+    const int64_t bx = cdiv(tpr, bdx);
+    // up to about 48 CTAs per SM, so that the last wave is short (1024 x 1M
+    // BF16: 362 us with 16, 348 with 48), but a chunk of 32 loads per thread or
+    // more (250 x 100,003 FP32, L = 1931: 50 us with shorter ones, 42)
+    int64_t kz = std::min(cdiv((int64_t)sms * 48, bx * M),
+                          std::max<int64_t>(1, grid_rows / ((int64_t)32 * bdy)));
+    kz = std::min<int64_t>(std::max<int64_t>(kz, 1), 65535);
     const int64_t kchunk = cdiv(grid_rows, kz);
     kz = cdiv(grid_rows, kchunk);
-    if (bx > 0x7fffffffLL || by > 65535) return cudaErrorInvalidValue;
-    dim3 grid((unsigned)bx, (unsigned)by, (unsigned)kz), block((unsigned)bdx, (unsigned)bdy);
-    if (dtype == KNN_BF16)
-      bin_max_mod_vec_kernel<KNN_BF16><<<grid, block, 0, st>>>(S, M, N, L, kchunk, neg, G);
-    else
-      bin_max_mod_vec_kernel<KNN_F32><<<grid, block, 0, st>>>(S, M, N, L, kchunk, neg, G);
-  } else if (bin_map == KNN_BINS_MOD) {
-    const int64_t grid_rows = cdiv(N, L);
-    const int64_t bx = cdiv(L, 256);
-    // enough CTAs to fill the GPU a few times over
-    int64_t kz = cdiv((int64_t)sms * 8, bx * M);
-    if (kz > grid_rows) kz = grid_rows;
-    if (kz < 1) kz = 1;
-    if (kz > 65535) kz = 65535;
-    const int64_t kchunk = cdiv(grid_rows, kz);
-    kz = cdiv(grid_rows, kchunk);
-    dim3 grid((unsigned)bx, (unsigned)M, (unsigned)kz);
-    if (dtype == KNN_BF16)
-      bin_max_mod_kernel<KNN_BF16><<<grid, 256, 0, st>>>(S, N, L, kchunk, neg, G);
-    else
-      bin_max_mod_kernel<KNN_F32><<<grid, 256, 0, st>>>(S, N, L, kchunk, neg, G);
+    if (bx > 0x7fffffffLL) return cudaErrorInvalidValue;
+    dim3 grid((unsigned)bx, (unsigned)M, (unsigned)kz), block((unsigned)bdx, (unsigned)bdy);
+    auto kern = dtype == KNN_BF16
+                    ? (vec ? bin_max_mod_kernel<KNN_BF16, 8> : bin_max_mod_kernel<KNN_BF16, 1>)
+                    : (vec ? bin_max_mod_kernel<KNN_F32, 4> : bin_max_mod_kernel<KNN_F32, 1>);
+    kern<<<grid, block, 0, st>>>(S, N, (int)L, (int)kchunk, neg, G);
   } else {
     const bool vec = N % vcols == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0;
     // columns per CTA: 32 vectors per thread, or 32 columns per thread

@@ -90,3 +90,24 @@ def test_approx_max_k_16_byte_loads_match_oracle(bins, dtype, N):
                 v, i = v.cpu().numpy(), i.cpu().numpy()
                 assert np.array_equal(i, oi), (L, is_min, agg)
                 assert np.array_equal(v.astype(np.float64), ov), (L, is_min, agg)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("M,N,L", [(3, 1, 1), (2, 9, 8), (5, 4096, 8), (7, 40_003, 1), (3, 40_000, 176),
+                                   (2, 100_003, 1931), (4, 65_536, 2048), (2, 70_000, 2064),
+                                   (1, 300_007, 255), (1, 300_000, 40)])
+def test_approx_max_k_grid_rows(M, N, L, dtype):
+    """Bin winners where the kernel's threads share a grid row's vectors and
+    several grid rows: few and many bins, 16-byte loads and single ones, a
+    ragged last grid row, more vectors than one block's threads."""
+    ensure_built()
+    X = scores(M, N, 43 + L)
+    t = torch.from_numpy(X).cuda()
+    if dtype == "bf16":
+        t = t.to(torch.bfloat16)
+    Xo = t.float().cpu().numpy().astype(np.float64)
+    for is_min in (False, True):
+        v, i = S.approx_max_k(t, 1, L=L, is_min=is_min, aggregate_to_topk=False)
+        ov, oi = oracle.approx_max_k(Xo, 1, L, is_min=is_min, aggregate_to_topk=False)
+        assert np.array_equal(i.cpu().numpy(), oi)
+        assert np.array_equal(v.cpu().numpy().astype(np.float64), ov)
