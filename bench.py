@@ -478,15 +478,15 @@ def main():
     # per-kernel times from the library's event profiler, in a separate pass
     # (its events are not part of the timed steps above)
     prof = profiled(lib, step, min(args.steps, 20))
-    # prep, K1 (plus the ragged-row kernel when N mod L != 0), then K2 and K3,
-    # or one launch of both when the library fuses them (no K3 launches)
+    # prep, K1, then K2 and K3, or one launch of both when the library fuses
+    # them (no K3 launches)
     fused23 = prof["k3"]["launches"] == 0
     kernels = {"prep": prof["prep"], "k1_partial_reduce": prof["k1"]}
     if fused23:
         kernels["k2_k3_rescoring_rerank_fused"] = prof["k2"]
     else:
         kernels["k2_rescoring"], kernels["k3_rerank"] = prof["k2"], prof["k3"]
-    launches_per_step = (3 if fused23 else 4) + (1 if bins == "mod" and N % L else 0)
+    launches_per_step = 3 if fused23 else 4
     S.sync_status()
 
     # the same step replayed from a CUDA graph (knn_search allocates nothing,
@@ -582,7 +582,7 @@ def main():
             "peak_source": "%s bf16 dense burst (MEASURED_PEAKS.json)" % pk_kind,
             "kernel": ("k1_tcs_kernel: fused BF16 contraction + PartialReduce, contiguous bins"
                        if bins == "contiguous" else
-                       "k1_tcs_kernel (+ k1_tcs_tail for the N mod L ragged rows): fused BF16 "
+                       "k1_tcs_kernel: fused BF16 "
                        "contraction + PartialReduce, j mod L bins"),
             "algorithmic": "2*M*N*D = %.4g FLOP per launch" % flops,
             "eq6": dict(eq6(M, N, D, k1_ms / 1e3, peak * 1e12, pk["hbm_gbs"] * 1e9,
@@ -719,10 +719,9 @@ def shard_main(args, world, rank, local):
                           "ms_per_step": job_ms / args.steps, "higher_is_better": True,
                           "scaling": "strong", "vs_baseline": None, "dtype": w["dtype"],
                           "data": "synthetic", "config": cfg, "recall_at_10": recall,
-                          # per step: prep, K1 (+ ragged rows), bin merge, key conversion;
-                          # key conversion, K2, FP32 scoring; key conversion, K2, pairs
-                          "gpu_launches": args.steps * (10 + (1 if n % L else 0) +
-                                                        (1 if metric == "cos" else 0)),
+                          # per step: prep, K1, bin merge, key conversion; key
+                          # conversion, K2, FP32 scoring; key conversion, K2 with its pairs
+                          "gpu_launches": args.steps * (9 + (1 if metric == "cos" else 0)),
                           "clocks": clk}))
     if world > 1:
         dist.destroy_process_group()

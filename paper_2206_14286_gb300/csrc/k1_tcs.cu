@@ -1143,17 +1143,20 @@ cudaError_t launch_k1_tcs(int64_t N, int64_t M, int64_t L, int D, int metric, in
   a.steps_per_q = runs ? cdiv(N, kCols) : grid;
   // One or two query halves per tile: a step costs its halves' MMAs, so one
   // half is taken where the halves do not pair up (M <= 128, or 333 queries: 3
-  // halves instead of 2 x 2). With one half every step is read from L2 for
-  // 128 queries instead of 256, counted as a tenth of its time. On 1M x 128 rows
-  // (L2) a search of 1, 128 and 333 queries took 61, 74 and 113 us with two
-  // halves and takes 51, 55 and 101 us; 64 queries on 4M x 768 rows 2.0 ms and
-  // 0.95 ms (6.5 TB/s).
+  // halves instead of 2 x 2). With one half every step is read from L2 for 128
+  // queries instead of 256, counted as a tenth of its time; with contiguous
+  // bins the epilogue also meets every bin in four warpgroups, which counts as
+  // half of it (333 queries on 700,001 x 100 rows, L2: 118 us with one half, 106
+  // with two; bins mod L: 90 and 110). On 1M x 128 rows (L2) a search of 1, 128
+  // and 333 queries took 61, 74 and 113 us with two halves and takes 51, 55 and
+  // 101 us; 64 queries on 4M x 768 rows 2.0 ms and 0.95 ms (6.5 TB/s).
   const int64_t sms = device_sm_count();
   int64_t kq1 = 1, parts1 = 1, spp1 = 1, groups1 = 1;
   tcs_schedule(cdiv(M, 2 * kQH), a.steps_per_q, sms, &a.kq, &a.parts, &a.steps_per_part, &a.groups);
   tcs_schedule(cdiv(M, kQH), a.steps_per_q, sms, &kq1, &parts1, &spp1, &groups1);
   int nh = 2;
-  if (1.1 * (double)kq1 * (double)(spp1 + 1) < 2.0 * (double)a.kq * (double)(a.steps_per_part + 1)) {
+  if ((runs ? 1.5 : 1.1) * (double)kq1 * (double)(spp1 + 1) <
+      2.0 * (double)a.kq * (double)(a.steps_per_part + 1)) {
     nh = 1;
     a.kq = kq1;
     a.parts = parts1;
