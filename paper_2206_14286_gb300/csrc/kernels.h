@@ -39,7 +39,7 @@ struct K1Plan {
 //                 0 marks a bin no row reached. The array must start at zero.
 struct Partials {
   float* v;         // packed / merged keys, 64-bit keys, or plain scores
-  int64_t index_offset;  // added to every decoded index (chunked exact search)
+  int64_t index_offset;  // added to every decoded index (a shard's first row)
   bool merged;
   bool keys64;      // v holds [M][L] 64-bit (score, ~index) keys, 0 = empty
 };
