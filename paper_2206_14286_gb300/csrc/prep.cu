@@ -71,10 +71,19 @@ __device__ __forceinline__ void add_square(Triple& a, float v) {
   a.m = __fadd_rn(a.m, r);
 }
 
-// Magnitudes for which the pairs behave: squares and their error terms
-// neither overflow nor lose bits that matter against the sum of the row's
-// squares. Anything else (zero rows too) takes the FP64 way.
-__device__ __forceinline__ bool pair_range(float mx) { return mx >= 0x1p-40f && mx <= 0x1p50f; }
+// Magnitudes for which the pairs behave (anything else, zero rows too, takes
+// the FP64 way). square_range: squares and their error terms neither overflow
+// nor lose bits that matter against the sum of the row's squares. unit_range,
+// for the inverse norm: its square, at least 2^(-2 kUnitHi) / kMaxD, is also
+// held exactly as two FP32 numbers: its last bit, 2^-48 of it, is no smaller
+// than FP32's smallest number, 2^-149. (With elements up to 2^50 that bit was
+// lost, and 1 / |x| was off by up to 2^-41 at D = 1024.)
+constexpr int kUnitHi = 40;
+static_assert(2 * kUnitHi + 48 <= 149 - 12 && kMaxD <= 1 << 12, "1 / |x|^2 loses bits");
+__device__ __forceinline__ bool square_range(float mx) { return mx >= 0x1p-40f && mx <= 0x1p50f; }
+__device__ __forceinline__ bool unit_range(float mx) {
+  return mx >= 0x1p-40f && mx <= (float)(1ll << kUnitHi);
+}
 
 // Sum over the G lanes of a row's group (G a power of two, groups aligned).
 template <int G>
@@ -127,9 +136,10 @@ __device__ __forceinline__ bool group_any(bool p) {
 
 // 1 / sqrt(n.h + n.l) as a pair: one Newton step from the hardware's
 // reciprocal square root y (relative error below 2^-22), the residual
-// 1 - n y^2 evaluated with error-free products. Terms of the residual are
-// below 2^-21 and round by 2^-24 of that; the cubic term left out is below
-// 2^-66: relative error below 2^-43.
+// 1 - n y^2 evaluated with error-free products (unit_range keeps y^2's two
+// parts out of the subnormals). Terms of the residual are below 2^-21 and
+// round by 2^-24 of that; the cubic term left out is below 2^-66: relative
+// error below 2^-43.
 __device__ __forceinline__ Pair inv_sqrt(float nh, float nl) {
   const float y = rsqrtf(nh);
   const float a = __fmul_rn(y, y), b = __fmaf_rn(y, y, -a);  // y^2 = a + b
@@ -271,7 +281,7 @@ __device__ __forceinline__ RowNorm norm_of(const float* xr, int D, bool vec, Row
   const float h = two_sum(s.h, __fadd_rn(s.l, s.m), e);
   n.inv = inv_sqrt(h, e);
   n.inv64 = 0.0;
-  bool undecided = !pair_range(mx) || !(h <= 3.0e38f);
+  bool undecided = !unit_range(mx) || !(h <= 3.0e38f);
 #pragma unroll
   for (int t = 0; t < nv; ++t) {
     float v[4];
@@ -511,7 +521,7 @@ prep_rows_kernel(const float* __restrict__ x, int64_t rows, int D, int pitch, in
     smx = group_max<G>(smx);
     const float m = __fmul_rn(h2.h, VPL > 0 ? 0x1p-35f : 0x1p-31f);
     const float up = __fadd_rn(h2.h, __fadd_rn(h2.l, m)), dn = __fadd_rn(h2.h, __fsub_rn(h2.l, m));
-    const bool open = !(up == dn && pair_range(smx));
+    const bool open = !(up == dn && square_range(smx));
     float hn = 0.5f * up;
     if (group_any<32>(open && live)) {
       double a = 0.0;

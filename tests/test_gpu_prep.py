@@ -92,3 +92,58 @@ def test_prepare_infinities_and_nan(D):
             t = torch.bfloat16 if dtype == "bf16" else torch.float32
             lp = d.lp.view(t).reshape(rows, d.pitch).float().cpu().numpy()
             assert (lp[:, D:] == 0).all()
+
+
+# 1024-element rows of 1022 times 2^50, then w 2^26, then v 2^7, (w, v) below:
+# the inverse norm's square is so small that FP32 holds it in a subnormal's few
+# bits, and v times the inverse norm lies within 2^-44 of a rounding midpoint,
+# so paired FP32 that took the inverse for good here rounds v to the other side
+# (found by exact evaluation of its steps). The hardware's reciprocal square
+# root may be off by a few units in the last place; rows for each.
+NEAR_2_50 = [
+    # off by -2 units in the last place
+    (0xee2d69, 0x85bacf), (0xee2d69, 0xa39114), (0xeb7ac2, 0x9bd93c), (0xeb7ac2, 0xbaab52), (0xd3772e, 0x9a354b),
+    (0xd3772e, 0xde10e1), (0xd411cd, 0x90af9d), (0xd411cd, 0x9eaed1), (0xbe7dea, 0x842046), (0xbe7dea, 0x90b5a2),
+    # off by -1 units in the last place
+    (0xf93989, 0xa4beec), (0xf93989, 0xc862f5), (0xcf3c70, 0xb91e72), (0x91b8d6, 0xd28106), (0xcae018, 0xa8d3c8),
+    (0xcae018, 0xc9c0ca), (0xec993f, 0xa87206), (0xb20fe8, 0xdb1b11), (0xb20fe8, 0xf5c456), (0xcdffbc, 0xfd28ee),
+    # off by 0 units in the last place
+    (0xb4f2af, 0xcb9648), (0xc33596, 0xd6b008), (0xa576bb, 0x9de3c2), (0x89a947, 0xdb5854), (0x89a947, 0xdc1323),
+    (0x96160a, 0xa212cf), (0x96160a, 0xe97ea6), (0xfac950, 0xb4242a), (0x89a915, 0xfe3051), (0xc33574, 0x91f5c1),
+    # off by 1 units in the last place
+    (0xf8472b, 0xfa6668), (0x80272e, 0x8474ab), (0x99866a, 0xeb1e4b), (0xa58ae2, 0xa277c8), (0xa58ae2, 0xb61a0e),
+    (0xdec760, 0x8531d7), (0xdec760, 0xfaf361), (0xf94e31, 0xf2c1d0), (0xfee1f8, 0xd30530), (0xfee1f8, 0xe6072d),
+    # off by 2 units in the last place
+    (0xe7ce45, 0x876d2e), (0xe7ce45, 0x8d091f), (0xf746ac, 0xfe53cd), (0x8e5db9, 0x937372), (0x8e5db9, 0xe15f1c),
+    (0xca616d, 0x82b7a9), (0xca616d, 0xa1356d), (0x8f42a5, 0x8a9d57), (0x8f42a5, 0xcdbe42), (0x955ead, 0xceda8d),
+]
+
+
+def test_prepare_bits_of_huge_norms():
+    ensure_built()
+    X = np.full((len(NEAR_2_50), 1024), 2.0 ** 50, np.float32)
+    X[:, 1022] = [w * 2.0 ** 26 for w, _ in NEAR_2_50]
+    X[:, 1023] = [v * 2.0 ** 7 for _, v in NEAR_2_50]
+    unit = oracle.normalize_rows(X)
+    for dtype in ("f32", "bf16", "e4m3"):
+        d = S.Database(torch.from_numpy(X).cuda(), metric="cos", dtype=dtype)
+        np.testing.assert_array_equal(d.f32.cpu().numpy().view(np.uint32), unit.view(np.uint32))
+
+
+@pytest.mark.parametrize("D", [64, 257, 1024, 1500, 4096])
+def test_prepare_bits_at_the_ends_of_the_paired_range(D):
+    """Rows whose largest element is at, just inside and just outside each end
+    of the range that paired FP32 handles (2^-40 and 2^40)."""
+    ensure_built()
+    g = np.random.Generator(np.random.PCG64(D))
+    tops = [np.float32(2.0 ** e) for e in (-41, -40, -39, 39, 40, 41, 50)]
+    tops += [np.nextafter(t, np.float32(s)) for t in tops for s in (0.0, np.inf)]
+    X = (g.uniform(0.5, 1.0, (16 * len(tops), D)) * g.choice([-1.0, 1.0], (16 * len(tops), D)))
+    X = (X * np.repeat(np.array(tops, np.float64), 16)[:, None]).astype(np.float32)
+    X[:, 0] = np.repeat(np.array(tops, np.float32), 16)
+    unit = oracle.normalize_rows(X)
+    d = S.Database(torch.from_numpy(X).cuda(), metric="cos", dtype="f32")
+    np.testing.assert_array_equal(d.f32.cpu().numpy().view(np.uint32), unit.view(np.uint32))
+    d = S.Database(torch.from_numpy(X).cuda(), metric="l2", dtype="f32")
+    X64 = X.astype(np.float64)
+    np.testing.assert_array_equal(d.hnorm.cpu().numpy(), (0.5 * (X64 * X64).sum(1)).astype(np.float32))
