@@ -369,6 +369,7 @@ size_t knn_partial_reduce_workspace(int64_t N, int32_t D, int32_t dtype, int32_t
  *                 the best K bin winners, best first.
  *   workspace   : knn_approx_max_k_workspace(...) bytes, 256-byte aligned.
  * Values are the scores as given (same sign); ties keep the smaller column.
+ * A NaN score comes before every other one, for the smallest scores too.
  * Reads every score once: HBM-bound. Errors: KNN_EINVAL (sizes, K > L with
  * aggregation, NULL, alignment, N >= 2^31), KNN_ENOMEM (workspace).
  */

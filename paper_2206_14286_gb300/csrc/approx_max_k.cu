@@ -28,11 +28,30 @@ __device__ __forceinline__ float load_score(const void* S, int64_t t, float sg) 
   return sg * v + 0.0f;
 }
 
+// The larger of two scores of load_score's form, a NaN above every other, and
+// whether it is not `a` (by its bits: a score of that form has one NaN, the
+// arithmetic's canonical positive one, and one zero).
+__device__ __forceinline__ float max_nan(float a, float b, bool& changed) {
+  float m;
+  asm("max.NaN.f32 %0, %1, %2;" : "=f"(m) : "f"(a), "f"(b));
+  changed = __float_as_uint(m) != __float_as_uint(a);
+  return m;
+}
+// make_key of a score, a NaN's too. (On the bits of a float the compiler turns
+// make_key's "| 0x80000000" into a negation, which loses a NaN's bits: a NaN
+// came out as -0. The empty asm makes them an integer's.)
+__device__ __forceinline__ uint64_t score_key(float v, int32_t j) {
+  uint32_t u = __float_as_uint(v);
+  asm("" : "+r"(u));
+  return ((uint64_t)((u & 0x80000000u) ? ~u : (u | 0x80000000u)) << 32) | (uint32_t)~j;
+}
+
 // Bins j mod L: a thread owns V bins b0 .. b0 + V - 1 of a row and walks their
 // columns, every bdy-th grid row of the CTA's chunk of grid rows, keeping each
-// bin's best value and grid row in registers (strict '>' while the column
-// grows keeps the smaller column on ties). V = 8 BF16 or 4 FP32 columns of one
-// 16-byte load (L and N multiples of V, S 16-byte aligned), else V = 1.
+// bin's best value and grid row in registers (a later column leads only by a
+// larger score, which keeps the smaller column on ties). V = 8 BF16 or 4 FP32
+// columns of one 16-byte load (L and N multiples of V, S 16-byte aligned), else
+// V = 1.
 //
 // Bound by HBM. threadIdx.x runs over the vectors of a grid row, however many
 // there are (tpr of them, up to 256), and threadIdx.y over grid rows, so the
@@ -40,8 +59,11 @@ __device__ __forceinline__ float load_score(const void* S, int64_t t, float sg) 
 // lane idles for padding: rounded up to warps, 22 vectors of L = 176 left 10 of
 // 32 lanes without work (1024 x 1M BF16: 510 us). The bdy rows' bests merge in
 // shared memory before one atomicMax per bin.
+// CTAs to an SM (by registers; with four of V = 8, 1024 x 1M BF16 took 374 us,
+// with five 316).
+constexpr int mod_ctas(int V) { return V == 8 ? 5 : V == 4 ? 6 : 8; }
 template <int DT, int V>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, mod_ctas(V))
 bin_max_mod_kernel(const void* __restrict__ S, int64_t N, int L, int kchunk, int neg,
                    unsigned long long* __restrict__ G) {
   constexpr int kEsz = DT == KNN_BF16 ? 2 : 4, U = V == 1 ? 8 : 4;
@@ -53,18 +75,19 @@ bin_max_mod_kernel(const void* __restrict__ S, int64_t N, int L, int kchunk, int
   const uint32_t T = (uint32_t)((N + L - 1) / L);  // grid rows, the last one maybe ragged
   const uint32_t k0 = blockIdx.z * (uint32_t)kchunk, k1 = min(T, k0 + kchunk);
   const float sg = neg ? -1.0f : 1.0f;
+  // every grid row but the last is whole
+  const uint32_t kfull = live && (int64_t)(k1 - 1) * L + b0 + V <= N ? k1 : k1 - 1;
+  // the first column leads with -inf until a score is larger
+  const bool any = live && k0 + threadIdx.y < kfull;
   float bv[V];
-  uint32_t bk[V], bo = 0;  // V = 1: the best score in the keys' order (NaN above all)
-  constexpr uint32_t kNone = 0xffffffffu;
+  uint32_t bk[V];
 #pragma unroll
   for (int c = 0; c < V; ++c) {
     bv[c] = neg_inf();
-    bk[c] = kNone;
+    bk[c] = k0 + threadIdx.y;
   }
-  if (live) {
+  if (any) {
     const char* row = static_cast<const char*>(S) + (i * N + b0) * kEsz;
-    // every grid row but the last is whole
-    const uint32_t kfull = (int64_t)(k1 - 1) * L + b0 + V <= N ? k1 : k1 - 1;
     auto take = [&](const uint4& raw, float one, uint32_t k) {
       float x[V];
       if constexpr (V == 1) {
@@ -82,16 +105,9 @@ bin_max_mod_kernel(const void* __restrict__ S, int64_t N, int L, int kchunk, int
       for (int c = 0; c < V; ++c) {
         // adding +0 turns -0 into +0: the two zeros tie
         const float v = sg * x[c] + 0.0f;
-        if constexpr (V == 1) {
-          const uint32_t o = float_to_ordered(v);
-          if (o > bo) {
-            bo = o;
-            bk[c] = k;
-          }
-        } else if (bk[c] == kNone || v > bv[c]) {
-          bv[c] = v;
-          bk[c] = k;
-        }
+        bool lead;
+        bv[c] = max_nan(bv[c], v, lead);
+        if (lead) bk[c] = k;
       }
     };
     auto load = [&](uint32_t k, uint4& raw, float& one) {
@@ -118,9 +134,7 @@ bin_max_mod_kernel(const void* __restrict__ S, int64_t N, int L, int kchunk, int
     }
   }
   auto key = [&](int c) -> uint64_t {
-    if (bk[c] == kNone) return (uint64_t)0;
-    const int32_t j = (int32_t)(bk[c] * (uint32_t)L + b0 + c);
-    return V == 1 ? ((uint64_t)bo << 32) | (uint32_t)~j : make_key(bv[c], j);
+    return any ? score_key(bv[c], (int32_t)(bk[c] * (uint32_t)L + b0 + c)) : (uint64_t)0;
   };
   if (bdy == 1) {
 #pragma unroll
@@ -188,7 +202,7 @@ bin_max_runs_kernel(const void* __restrict__ S, int64_t N, int64_t L, int64_t ch
           end = (cur + 1) * q + min(cur + 1, r);
           best = 0;
         }
-        const uint64_t key = make_key(v[u], (int32_t)j);
+        const uint64_t key = score_key(v[u], (int32_t)j);
         best = key > best ? key : best;
       }
     }
@@ -215,7 +229,7 @@ bin_max_runs_vec_kernel(const void* __restrict__ S, int64_t N, int64_t L, int64_
   float bv = neg_inf();
   int32_t bj = -1;
   auto flush = [&]() {
-    if (bj >= 0) atomicMax(&G[i * L + cur], (unsigned long long)make_key(bv, bj));
+    if (bj >= 0) atomicMax(&G[i * L + cur], (unsigned long long)score_key(bv, bj));
   };
   const int64_t step = (int64_t)blockDim.x * V;
   for (int64_t jv = j0 + (int64_t)threadIdx.x * V; jv < j1; jv += 4 * step) {
@@ -248,13 +262,12 @@ bin_max_runs_vec_kernel(const void* __restrict__ S, int64_t N, int64_t L, int64_
             cur = runs_bin_of(jj, q, r);
             end = (cur + 1) * q + min(cur + 1, r);
             bv = neg_inf();
-            bj = -1;
-          }
-          const float v = sg * x[c] + 0.0f;
-          if (bj < 0 || v > bv) {
-            bv = v;
             bj = (int32_t)jj;
           }
+          const float v = sg * x[c] + 0.0f;
+          bool lead;
+          bv = max_nan(bv, v, lead);
+          if (lead) bj = (int32_t)jj;
         }
       }
     }

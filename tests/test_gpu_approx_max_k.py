@@ -111,3 +111,43 @@ def test_approx_max_k_grid_rows(M, N, L, dtype):
         ov, oi = oracle.approx_max_k(Xo, 1, L, is_min=is_min, aggregate_to_topk=False)
         assert np.array_equal(i.cpu().numpy(), oi)
         assert np.array_equal(v.cpu().numpy().astype(np.float64), ov)
+
+
+@pytest.mark.parametrize("bins", ["mod", "contiguous"])
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+def test_approx_max_k_nan_comes_first(bins, dtype):
+    """One rule for NaN (before every other score, the smaller column among
+    several), the same with 16-byte loads and with single ones (the matrix
+    starting one element later): NaN in the first, a middle and the last grid
+    row of a bin, twice in a bin, beside infinities, and bins of -inf alone."""
+    ensure_built()
+    M, N = 4, 8192
+    g = np.random.Generator(np.random.PCG64(51))
+    X = g.standard_normal((M, N)).astype(np.float32)
+    X[0, [3, 4099, 8191]] = np.nan
+    X[1, [100, 101, 4000, 4001, 5000]] = [np.nan, np.inf, np.inf, np.nan, -np.inf]
+    X[2, :] = -np.inf
+    X[2, [7, 4103]] = np.nan
+    X[3, :] = np.inf
+    X[3, 8000] = np.nan
+    flat = torch.empty(M * N + 1, device="cuda")
+    flat[1:] = torch.from_numpy(X).cuda().reshape(-1)
+    if dtype == "bf16":
+        flat = flat.to(torch.bfloat16)
+    shifted = flat[1:].view(M, N)
+    Xo = shifted.float().cpu().numpy().astype(np.float64)
+    for is_min in (False, True):
+        rank = np.clip(-Xo if is_min else Xo, -1e200, 1e200)
+        rank[np.isnan(Xo)] = 1e300
+        for L in (8, 64, 176, 4096, N):
+            j = np.arange(N)
+            q, r = N // L, N % L
+            b = j % L if bins == "mod" else np.where(j < r * (q + 1), j // (q + 1),
+                                                     r + (j - r * (q + 1)) // q)
+            first = np.array([[np.flatnonzero(b == t)[np.argmax(rank[i, b == t])]
+                               for t in range(L)] for i in range(M)])
+            for t in (shifted, shifted.clone()):
+                v, i = S.approx_max_k(t, 1, L=L, bins=bins, is_min=is_min, aggregate_to_topk=False)
+                np.testing.assert_array_equal(i.cpu().numpy(), first)
+                np.testing.assert_array_equal(v.cpu().numpy().astype(np.float64),
+                                              np.take_along_axis(Xo, first, 1))
