@@ -102,7 +102,9 @@ class Database:
     def _search_plan(self, M, K, L, recall_target, rerank, bins):
         """(bins, workspace bytes) of a search with these sizes: a function of
         the arguments alone, kept for the sizes that come again."""
-        key = (M, K, L, recall_target, rerank, bins)
+        # by value: an argument may be a tensor or an array element, which later
+        # holds another number under the same identity
+        key = (int(M), int(K), int(L) if L else 0, float(recall_target), int(rerank), bins)
         plan = self._plans.get(key)
         if plan is None:
             Lr = self.resolve_L(K, L, recall_target)
