@@ -5,8 +5,8 @@
 // One CTA per query holds its L <= 8192 keys in registers. Up to Kp = 128 the
 // Kp-th largest of the 256 threads' maxima bounds the selection from below:
 // few keys beyond Kp reach it, and those are gathered and sorted. Larger Kp: a
-// radix select. More candidates (L > 8192, or Kp > 1024) stream through
-// shared memory against the running Kp-th best key.
+// radix select. What is left streams through shared memory against the running
+// Kp-th best key: more candidates (L > 8192), or a sorted selection of Kp > 1024.
 #include <algorithm>
 
 #include "common.cuh"
@@ -428,8 +428,9 @@ __device__ __forceinline__ void sort_buf(uint64_t* buf, int c, int fill) {
   bitonic_sort_desc(buf, P2);
 }
 
-// The best Kp <= kTopkCap of the CTA's L keys (thread t holds keys t + 256 u)
-// into sm.buf[0..Kp): sorted best first if `sorted`, else as a set.
+// The best Kp of the CTA's L keys (thread t holds keys t + 256 u) into
+// dst[0..Kp): sorted best first if `sorted`, else as a set. dst is sm.buf for
+// Kp <= kTopkCap; more keys, as a set only, go to global memory.
 //
 // Up to kThrMaxK: the Kp-th largest of the threads' maxima (high words) is a
 // lower bound of the Kp-th largest key; the keys that reach it are gathered.
@@ -439,7 +440,7 @@ __device__ __forceinline__ void sort_buf(uint64_t* buf, int c, int fill) {
 // are distinct but for empty ones (0), so the set is that of a sort.
 template <int KPT>
 __device__ __forceinline__ void select_topk(const uint64_t (&k)[KPT], int L, int Kp, bool sorted,
-                                            SelectSmem& sm) {
+                                            SelectSmem& sm, uint64_t* dst) {
   const int tid = threadIdx.x, lane = tid & 31;
   bool radix = Kp > kThrMaxK;
   if (tid == 0) sm.cnt = 0;
@@ -499,13 +500,13 @@ __device__ __forceinline__ void select_topk(const uint64_t (&k)[KPT], int L, int
     if (u * 256 + tid >= L) continue;
     const uint64_t m = k[u] & mask;
     if (m > prefix) {
-      sm.buf[atomicAdd(&sm.cnt, 1)] = k[u];
+      dst[atomicAdd(&sm.cnt, 1)] = k[u];
     } else if (m == prefix) {
       const int p = atomicAdd(&sm.above, 1);
-      if (p < need) sm.buf[n_hi + p] = k[u];
+      if (p < need) dst[n_hi + p] = k[u];
     }
   }
-  for (int t = L + tid; t < Kp; t += 256) sm.buf[t] = 0;  // Kp > L: empty
+  for (int t = L + tid; t < Kp; t += 256) dst[t] = 0;  // Kp > L: empty
   __syncthreads();
   if (sorted) sort_buf(sm.buf, Kp, Kp);
 }
@@ -520,9 +521,12 @@ __device__ __forceinline__ void load_keys(const Src& src, int64_t i, int L, uint
 }
 
 // ExactRescoring alone: the best Kp keys of each query, as keys or (out_val
-// given) as values, negated when `neg`, and indices.
+// given) as values, negated when `neg`, and indices. kDirect: more than kTopkCap
+// keys (a set for a re-rank) are written as they are gathered: 1000 queries, L =
+// 8192, 1600 candidates of 64 elements 375 us a search; the streaming kernel
+// below, whose sorted buffer holds them all, 1513.
 // (three CTAs per SM with up to 8192 keys: 10,000 queries 1.18 -> 0.86 ms)
-template <class Src, int KPT>
+template <class Src, int KPT, bool kDirect>
 __global__ void __launch_bounds__(256, KPT == 32 ? 3 : 4)
 k2_select_kernel(Src src, int L, int Kp, bool sorted, uint64_t* __restrict__ out_keys, int neg,
                  float* __restrict__ out_val, int32_t* __restrict__ out_idx) {
@@ -531,7 +535,11 @@ k2_select_kernel(Src src, int L, int Kp, bool sorted, uint64_t* __restrict__ out
   pdl_wait();
   uint64_t k[KPT];
   load_keys(src, i, L, k);
-  select_topk(k, L, Kp, sorted, sm);
+  if constexpr (kDirect) {
+    select_topk(k, L, Kp, false, sm, out_keys + i * Kp);
+    return;
+  }
+  select_topk(k, L, Kp, sorted, sm, sm.buf);
   for (int t = threadIdx.x; t < Kp; t += 256) {
     const uint64_t key = sm.buf[t];
     if (out_val) {
@@ -579,7 +587,7 @@ __global__ void __launch_bounds__(256) rescore_kernel(Src src, RescoreArgs a) {
   } else {
     uint64_t k[KPT];
     load_keys(src, i, a.L, k);
-    select_topk(k, a.L, a.Kp, false, sm);
+    select_topk(k, a.L, a.Kp, false, sm, sm.buf);
   }
   const float* q = a.qf32 + i * a.q_stride;
   constexpr int kCand = KPT == 0 ? 8 : 4;
@@ -668,7 +676,7 @@ __global__ void __launch_bounds__(256) rescore_kernel(Src src, RescoreArgs a) {
       k[u] = c < a.Kp ? sm.buf[c] : 0;
     }
     __syncthreads();
-    select_topk(k, a.Kp, a.K, true, sm);
+    select_topk(k, a.Kp, a.K, true, sm, sm.buf);
   }
   for (int t = tid; t < a.K; t += 256) {
     const uint64_t key = sm.buf[t];
@@ -682,10 +690,14 @@ __global__ void __launch_bounds__(256) rescore_kernel(Src src, RescoreArgs a) {
 template <class Src>
 cudaError_t run_k2_select(const Src& src, int64_t M, int64_t L, int Kp, bool sorted, uint64_t* out,
                           int neg, float* out_val, int32_t* out_idx, cudaStream_t st) {
-  auto kern = L <= 1024   ? k2_select_kernel<Src, 4>
-              : L <= 2048 ? k2_select_kernel<Src, 8>
-              : L <= 4096 ? k2_select_kernel<Src, 16>
-                          : k2_select_kernel<Src, 32>;
+  auto kern = L <= 1024   ? k2_select_kernel<Src, 4, false>
+              : L <= 2048 ? k2_select_kernel<Src, 8, false>
+              : L <= 4096 ? k2_select_kernel<Src, 16, false>
+                          : k2_select_kernel<Src, 32, false>;
+  if (Kp > kTopkCap)
+    kern = L <= 2048   ? k2_select_kernel<Src, 8, true>
+           : L <= 4096 ? k2_select_kernel<Src, 16, true>
+                       : k2_select_kernel<Src, 32, true>;
   return launch_pdl(kern, dim3((unsigned)M), dim3(256), 0, st, src, (int)L, Kp, sorted, out, neg,
                     out_val, out_idx);
 }
@@ -821,12 +833,12 @@ block_topk_kernel(Src src, int64_t n, int64_t nblk, int K, uint64_t* __restrict_
 
 }  // namespace
 
-// Per query: one CTA with the candidates in registers up to 8192 of them and
-// 1024 selected; the streaming CTA kernel everything else.
+// Per query: one CTA with the candidates in registers up to 8192 of them, and
+// 1024 selected if they are to be sorted; the streaming CTA kernel everything else.
 template <class Src>
 cudaError_t dispatch_k2(const Src& s, const K1Plan& p, int Kp, uint64_t* out_keys, bool sorted,
                         cudaStream_t st) {
-  if (p.L <= kTopkElems && Kp <= kTopkCap && p.M <= 0x7fffffffLL)
+  if (p.L <= kTopkElems && (Kp <= kTopkCap || !sorted) && p.M <= 0x7fffffffLL)
     return run_k2_select(s, p.M, p.L, Kp, sorted, out_keys, 0, nullptr, nullptr, st);
   return run_k2(s, p.M, p.L, Kp, nullptr, out_keys, st);
 }

@@ -57,3 +57,49 @@ def test_rescored_search(metric, N):
             rv, ri = ranked(s, K)
             assert torch.equal(idx.long(), ri)
             assert torch.equal(val, -rv if metric == "l2" else rv)
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16", "e4m3"])
+@pytest.mark.parametrize("N", [1025, 2048, 2049, 4096, 4097, 8192])
+def test_rescored_search_of_many_candidates(N, dtype):
+    """Re-ranks of more than 1024 candidates, every row its own bin: the exact
+    top-K, at the edges of the selection's keys per thread."""
+    ensure_built()
+    D = 20
+    x, q = ints((N, D), N, -2, 3), ints((9, D), D, -2, 3)
+    if dtype == "e4m3":                       # scales 1: codes are the values
+        x[:, 0], q[:, 0] = 448.0, 448.0
+    d = S.Database(x, metric="ip", dtype=dtype)
+    s = q @ x.t()
+    for K, r in ((1, 1025), (1025, 1), (200, 6), (200, 8), (1024, 4), (N, 1)):
+        if K > min(N, 4096):
+            continue
+        val, idx = d.search(q, K, L=N, rerank=r)
+        rv, ri = ranked(s, K)
+        assert torch.equal(idx.long(), ri)
+        assert torch.equal(val, rv)
+
+
+def test_selection_of_more_than_1024_candidates_stays_a_selection():
+    """One candidate more than the selection's buffer holds must not send the
+    call to a sort of everything (4 times the call, measured)."""
+    ensure_built()
+    x, q = ints((8192, 16), 1, -2, 3), ints((2000, 16), 2, -2, 3)
+    d = S.Database(x, metric="ip", dtype="bf16")
+
+    def us(K, r):
+        for _ in range(3):
+            d.search(q, K, L=8192, rerank=r)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        t = []
+        for _ in range(15):
+            a.record()
+            d.search(q, K, L=8192, rerank=r)
+            b.record()
+            b.synchronize()
+            t.append(a.elapsed_time(b))
+        return min(t)
+
+    # a quarter more candidates to gather and sort; 2.2 leaves the re-rank of
+    # more than 1024 its sort of 2048 keys
+    assert us(205, 5) < 2.2 * us(128, 8)
