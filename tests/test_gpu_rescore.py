@@ -80,26 +80,51 @@ def test_rescored_search_of_many_candidates(N, dtype):
         assert torch.equal(val, rv)
 
 
+def us(d, q, K, L, r):
+    for _ in range(3):
+        d.search(q, K, L=L, rerank=r)
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    t = []
+    for _ in range(15):
+        a.record()
+        d.search(q, K, L=L, rerank=r)
+        b.record()
+        b.synchronize()
+        t.append(a.elapsed_time(b))
+    return min(t)
+
+
 def test_selection_of_more_than_1024_candidates_stays_a_selection():
     """One candidate more than the selection's buffer holds must not send the
     call to a sort of everything (4 times the call, measured)."""
     ensure_built()
     x, q = ints((8192, 16), 1, -2, 3), ints((2000, 16), 2, -2, 3)
     d = S.Database(x, metric="ip", dtype="bf16")
-
-    def us(K, r):
-        for _ in range(3):
-            d.search(q, K, L=8192, rerank=r)
-        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        t = []
-        for _ in range(15):
-            a.record()
-            d.search(q, K, L=8192, rerank=r)
-            b.record()
-            b.synchronize()
-            t.append(a.elapsed_time(b))
-        return min(t)
-
     # a quarter more candidates to gather and sort; 2.2 leaves the re-rank of
     # more than 1024 its sort of 2048 keys
-    assert us(205, 5) < 2.2 * us(128, 8)
+    assert us(d, q, 205, 8192, 5) < 2.2 * us(d, q, 128, 8192, 8)
+
+
+@pytest.mark.parametrize("M", [47, 48, 49, 151, 152, 607, 608, 609])
+def test_rescored_search_of_a_few_queries_per_sm(M):
+    """The numbers of queries around which the rescoring's launch changes."""
+    ensure_built()
+    for N in (1024, 4096):
+        x, q = ints((N, 24), N + M, -2, 3), ints((M, 24), M, -2, 3)
+        d = S.Database(x, metric="ip", dtype="bf16")
+        s = q @ x.t()
+        for K, r in ((10, 2), (100, 8)):
+            val, idx = d.search(q, K, L=N, rerank=r)
+            rv, ri = ranked(s, K)
+            assert torch.equal(idx.long(), ri)
+            assert torch.equal(val, rv)
+
+
+def test_rescoring_of_a_query_per_sm_does_not_crowd():
+    """A CTA per query, fewer queries than SMs: no more than one query takes,
+    give or take the contraction's larger tile (launched early, while the
+    contraction still held the SMs, they took twice as long)."""
+    ensure_built()
+    x, q = ints((60_000, 64), 3, -2, 3), ints((100, 64), 4, -2, 3)
+    d = S.Database(x, metric="l2", dtype="bf16")
+    assert us(d, q, 1024, 1024, 1) < 1.5 * us(d, q[:1], 1024, 1024, 1)
