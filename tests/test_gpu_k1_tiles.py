@@ -78,3 +78,51 @@ def test_partial_reduce_work_split(dtype, metric, M, N, L, D):
         own = s.gather(1, A)
         assert ((V.double() - own).abs() <= tol).all()     # the value is its row's score
         assert (best - own <= 2 * tol).all()               # and the bin's best
+
+
+def us(f):
+    for _ in range(3):
+        f()
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    t = []
+    for _ in range(11):
+        a.record()
+        f()
+        b.record()
+        b.synchronize()
+        t.append(a.elapsed_time(b))
+    return min(t)
+
+
+def test_fp32_tiles_of_a_cta_per_sm_spread_over_the_sms():
+    """144 CTAs of one tile each take no longer than 48 of them, give or take
+    their share of the memory system (two to an SM they took 1.6 times as long)."""
+    ensure_built()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(3)
+    x = torch.randn((3000, 4096), generator=g, device="cuda")
+    q = torch.randn((333, 4096), generator=g, device="cuda")
+    d = S.Database(x, metric="ip", dtype="f32")
+    assert us(lambda: d.partial_reduce(q, 1024)) < 1.3 * us(lambda: d.partial_reduce(q[:128], 1024))
+
+
+@pytest.mark.parametrize("M,N,L", [(333, 3000, 605), (1000, 3000, 1024), (65, 9000, 1024),
+                                   (70, 20_000, 2000), (7, 100, 3)])
+def test_fp32_partial_reduce_launches(M, N, L):
+    """The FP32 kernel's launches (an SM to each CTA, in order, early), on
+    integers: exact scores and the smaller row on ties."""
+    ensure_built()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M)
+    x = torch.randint(-2, 3, (N, 20), generator=g, device="cuda").float()
+    q = torch.randint(-2, 3, (M, 20), generator=g, device="cuda").float()
+    V, A = S.Database(x, metric="ip", dtype="f32").partial_reduce(q, L)
+    # the bins' columns side by side, -inf past the last row; the first maximum
+    T = (N + L - 1) // L
+    s = torch.full((M, T * L), -float("inf"), device="cuda")
+    s[:, :N] = q @ x.t()
+    s = s.view(M, T, L)
+    best = s.amax(1)
+    first = (s == best[:, None, :]).float().argmax(1)
+    assert torch.equal(V, best)
+    assert torch.equal(A.long(), first * L + torch.arange(L, device="cuda")[None, :])
