@@ -960,16 +960,28 @@ int64_t grid_steps(int64_t N, int64_t Lv, TcsArgs* a) {
 }
 
 // How many virtual bins per bin: the grids are padded to groups of 16 bins, so
-// few bins waste MMAs (L = 20: two groups of 16, 1.6x the steps).
-// The fold with the fewest steps, each further fold counted as one per cent
-// for its additional merges and position searches.
-int64_t pick_fold(int64_t N, int64_t L, int64_t row_bytes) {
+// few bins waste MMAs (L = 20: two groups of 16, 1.6x the steps). The fold with
+// the least time, in microseconds:
+//   - the steps of a CTA, 0.45 per K block and query half, each further fold
+//     counted as one per cent for its position searches;
+//   - the merges into fewer than 16 bins, which all CTAs make at once: with L = 3
+//     the 304 (CTA, accumulator) pairs of up to 128 queries add 5 ns for each
+//     virtual bin (60,000 x 64 rows, 64 queries: fold 1, 3, 5 took 22, 24, 45 us, and
+//     300,000 rows 45, 40, 56; 256 queries 24, 23, 30), more bins spread them over
+//     more lines (L = 5, 7, 10: 40, 30, 24 us at 16 virtual bins). Few queries have
+//     few merges (1 query: 19-20 us whatever the fold).
+int64_t pick_fold(int64_t N, int64_t L, int64_t row_bytes, int64_t M, int64_t sms) {
   int64_t best = 1;
   double cost = 0.0;
+  const double halves = (double)cdiv(M, kQH);
+  const double step = 0.45 * (double)cdiv(row_bytes, kSpanS) * halves / (double)sms;
+  const double merge = 0.005 * 2.0 * (double)sms / halves * std::min(1.0, 3.0 / (double)L) *
+                       std::min(1.0, (double)M / 64.0);
   for (int64_t f = 1; f <= 16; ++f) {
     if (f > 1 && (f * L * kRowsBin > N || f * L * row_bytes >= ((int64_t)1 << 40))) break;
     TcsArgs a{};
-    const double c = (double)grid_steps(N, f * L, &a) * (1.0 + 0.01 * (double)(f - 1));
+    const double c = (double)grid_steps(N, f * L, &a) * step * (1.0 + 0.01 * (double)(f - 1)) +
+                     merge * (double)std::min<int64_t>(f * L, kStepBins);
     if (f == 1 || c < cost) {
       best = f;
       cost = c;
@@ -1139,7 +1151,9 @@ cudaError_t launch_k1_tcs(int64_t N, int64_t M, int64_t L, int D, int metric, in
   a.bq = (uint32_t)(N / L);
   a.br = (uint32_t)(N % L);
   // a step: 16 bins x 16 grid rows (j mod L), or 256 consecutive rows
-  const int64_t grid = grid_steps(N, runs ? L : L * pick_fold(N, L, (int64_t)pitch * esz), &a);
+  const int64_t sms = std::max(1, device_sm_count());
+  const int64_t grid =
+      grid_steps(N, runs ? L : L * pick_fold(N, L, (int64_t)pitch * esz, M, sms), &a);
   a.steps_per_q = runs ? cdiv(N, kCols) : grid;
   // One or two query halves per tile: a step costs its halves' MMAs, so one
   // half is taken where the halves do not pair up (M <= 128, or 333 queries: 3
@@ -1150,7 +1164,6 @@ cudaError_t launch_k1_tcs(int64_t N, int64_t M, int64_t L, int D, int metric, in
   // with two; bins mod L: 90 and 110). On 1M x 128 rows (L2) a search of 1, 128
   // and 333 queries took 61, 74 and 113 us with two halves and takes 51, 55 and
   // 101 us; 64 queries on 4M x 768 rows 2.0 ms and 0.95 ms (6.5 TB/s).
-  const int64_t sms = device_sm_count();
   int64_t kq1 = 1, parts1 = 1, spp1 = 1, groups1 = 1;
   tcs_schedule(cdiv(M, 2 * kQH), a.steps_per_q, sms, &a.kq, &a.parts, &a.steps_per_part, &a.groups);
   tcs_schedule(cdiv(M, kQH), a.steps_per_q, sms, &kq1, &parts1, &spp1, &groups1);
