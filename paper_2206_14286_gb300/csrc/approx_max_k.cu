@@ -10,6 +10,7 @@
 // keep the smaller column whatever the order of the CTAs; approx_min_k
 // negates the scores on the way in and the values on the way out.
 #include <algorithm>
+#include <cmath>
 #include <cuda_bf16.h>
 
 #include "common.cuh"
@@ -58,20 +59,23 @@ __device__ __forceinline__ uint64_t score_key(float v, int32_t j) {
 // CTA's threads read bdy whole grid rows, which are adjacent in memory, and no
 // lane idles for padding: rounded up to warps, 22 vectors of L = 176 left 10 of
 // 32 lanes without work (1024 x 1M BF16: 510 us). The bdy rows' bests merge in
-// shared memory before one atomicMax per bin.
+// shared memory before one atomicMax per bin. kRows: threadIdx.z runs over rows
+// of S, where a row's columns are too few for more threads (an instance of its
+// own: with the row a thread's, not a CTA's, 250 x 100,003 FP32 was 3% slower).
 // CTAs to an SM (by registers; with four of V = 8, 1024 x 1M BF16 took 374 us,
 // with five 316).
 constexpr int mod_ctas(int V) { return V == 8 ? 5 : V == 4 ? 6 : 8; }
-template <int DT, int V>
+template <int DT, int V, bool kRows>
 __global__ void __launch_bounds__(256, mod_ctas(V))
-bin_max_mod_kernel(const void* __restrict__ S, int64_t N, int L, int kchunk, int neg,
+bin_max_mod_kernel(const void* __restrict__ S, int M, int64_t N, int L, int kchunk, int neg,
                    unsigned long long* __restrict__ G) {
   constexpr int kEsz = DT == KNN_BF16 ? 2 : 4, U = V == 1 ? 8 : 4;
   __shared__ uint64_t part[V == 1 ? 1 : V][256];
-  const int tid = threadIdx.y * blockDim.x + threadIdx.x, bdy = blockDim.y;
-  const int64_t i = blockIdx.y;
+  const int bdy = blockDim.y;
+  const int zt = kRows ? threadIdx.z * bdy * blockDim.x : 0;  // first thread of this row
+  const int64_t i = kRows ? (int64_t)blockIdx.y * blockDim.z + threadIdx.z : blockIdx.y;
   const int b0 = ((int)blockIdx.x * blockDim.x + threadIdx.x) * V;
-  const bool live = b0 < L;
+  const bool live = b0 < L && (!kRows || i < M);
   const uint32_t T = (uint32_t)((N + L - 1) / L);  // grid rows, the last one maybe ragged
   const uint32_t k0 = blockIdx.z * (uint32_t)kchunk, k1 = min(T, k0 + kchunk);
   const float sg = neg ? -1.0f : 1.0f;
@@ -144,20 +148,16 @@ bin_max_mod_kernel(const void* __restrict__ S, int64_t N, int L, int kchunk, int
     }
     return;
   }
+  const int t0 = threadIdx.y * blockDim.x + threadIdx.x;
 #pragma unroll
-  for (int c = 0; c < V; ++c) {
-    if constexpr (V == 1)
-      part[0][tid] = key(c);
-    else
-      part[c][tid] = key(c);
-  }
+  for (int c = 0; c < V; ++c) part[V == 1 ? 0 : c][zt + t0] = key(c);
   __syncthreads();
-  for (int t = tid; t < (int)blockDim.x * V; t += blockDim.x * bdy) {
+  for (int t = t0; t < (int)blockDim.x * V; t += blockDim.x * bdy) {
     const int c = t / blockDim.x, x = t % blockDim.x;
     const int b = ((int)blockIdx.x * blockDim.x + x) * V + c;
     uint64_t best = 0;
     for (int y = 0; y < bdy; ++y) {
-      const uint64_t o = part[c][y * blockDim.x + x];
+      const uint64_t o = part[c][zt + y * blockDim.x + x];
       best = o > best ? o : best;
     }
     if (best && b < L) atomicMax(&G[i * L + b], (unsigned long long)best);
@@ -275,6 +275,64 @@ bin_max_runs_vec_kernel(const void* __restrict__ S, int64_t N, int64_t L, int64_
   flush();
 }
 
+// How the columns of j mod L bins are shared out: a CTA takes the bdx vectors of
+// bdy grid rows at a time of bdz rows of S, kchunk grid rows of them, kz chunks
+// to a row.
+struct ModShape {
+  int bdx, bdy, bdz;
+  int64_t kz, kchunk;
+};
+// A thread has 32 loads or more before its CTA's bests merge, so few grid rows
+// are shared by few threads, and the CTA's other threads take other rows of S
+// (5000 x 4096 FP32, L = 128, 32 grid rows: 42 us a call with 8 threads over them,
+// 28 with 1; 20,000 x 1024, L = 8, 128 grid rows: 29.4 us with 8, 28.4 with 4).
+// The chunks: the time is the waves of CTAs times a chunk's loads per thread plus
+// about eight loads' time for its start and its merge. (With at least 32 loads
+// a chunk and up to 48 CTAs per SM, waves were left part empty: 3 x 20M FP32, L =
+// 8, 61 us with 610 chunks a row, 47 with 304; 500 x 65,536, L = 128: 44 and 34; and
+// one row of 1M BF16, L = 2064, had 30 CTAs.) More than 304 chunks queue for their
+// bins' keys: one row of 1M FP32, L = 128, 41 us with 869, 20 with 300 or fewer.
+ModShape mod_shape(int64_t M, int64_t grid_rows, int64_t tpr, int V) {
+  constexpr int64_t kLoads = 32, kEdge = 8, kMaxChunks = 304;
+  ModShape s;
+  s.bdx = (int)std::min<int64_t>(256, tpr);
+  const int64_t room = 256 / s.bdx;
+  s.bdy = (int)std::min(room, std::max<int64_t>(1, grid_rows / kLoads));
+  s.bdz = (int)std::min(std::min(room / s.bdy, M), (int64_t)64);
+  const int64_t warps = cdiv((int64_t)s.bdx * s.bdy * s.bdz, 32);
+  const int64_t slots = device_sm_count() * std::min<int64_t>(32, mod_ctas(V) * 8 / warps);
+  const int64_t ctas = cdiv(tpr, s.bdx) * cdiv(M, s.bdz);  // of one chunk
+  // chunk counts that end a wave; beyond two waves the CTAs no longer run in step,
+  // and about half a chunk is left over at the end (1024 x 1M BF16: 337 us with 2
+  // chunks a row, in 2.7 waves, 316 with 8, in 10.8)
+  double best = -1.0;
+  s.kz = 1;
+  s.kchunk = grid_rows;
+  const int64_t w0 = std::max<int64_t>(1, cdiv(ctas, slots));
+  for (int64_t w = w0; w < w0 + 12; ++w) {
+    const int64_t kz = std::min(std::min(w * slots / ctas, grid_rows), kMaxChunks);
+    const int64_t kchunk = cdiv(grid_rows, kz), n = cdiv(grid_rows, kchunk);
+    const double waves = (double)(ctas * n) / (double)slots;
+    const double cost = (waves <= 2.0 ? std::ceil(waves) : waves + 0.5) *
+                        (double)(cdiv(kchunk, s.bdy) + kEdge);
+    if (best < 0.0 || cost < best) {
+      best = cost;
+      s.kz = n;
+      s.kchunk = kchunk;
+    }
+    if (kz == grid_rows || kz == kMaxChunks) break;
+  }
+  return s;
+}
+
+template <bool kRows>
+auto mod_kernel(int dtype, bool vec) {
+  return dtype == KNN_BF16 ? (vec ? bin_max_mod_kernel<KNN_BF16, 8, kRows>
+                                  : bin_max_mod_kernel<KNN_BF16, 1, kRows>)
+                           : (vec ? bin_max_mod_kernel<KNN_F32, 4, kRows>
+                                  : bin_max_mod_kernel<KNN_F32, 1, kRows>);
+}
+
 // Keys to (value, index) pairs, values back in the caller's orientation.
 __global__ void keys_to_pairs_kernel(const uint64_t* __restrict__ keys, int64_t n, int neg,
                                      float* __restrict__ out_v, int32_t* __restrict__ out_a) {
@@ -307,23 +365,12 @@ cudaError_t launch_bin_max(const void* S, int dtype, int64_t M, int64_t N, int64
     const bool vec = L % vcols == 0 && N % vcols == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0;
     const int64_t tpr = vec ? L / vcols : L;  // threads that cover a grid row
     const int64_t grid_rows = cdiv(N, L);
-    const int bdx = (int)std::min<int64_t>(256, tpr);
-    const int bdy = (int)std::max<int64_t>(1, std::min<int64_t>(256 / bdx, grid_rows));
-    const int64_t bx = cdiv(tpr, bdx);
-    // up to about 48 CTAs per SM, so that the last wave is short (1024 x 1M
-    // BF16: 362 us with 16, 348 with 48), but a chunk of 32 loads per thread or
-    // more (250 x 100,003 FP32, L = 1931: 50 us with shorter ones, 42)
-    int64_t kz = std::min(cdiv((int64_t)sms * 48, bx * M),
-                          std::max<int64_t>(1, grid_rows / ((int64_t)32 * bdy)));
-    kz = std::min<int64_t>(std::max<int64_t>(kz, 1), 65535);
-    const int64_t kchunk = cdiv(grid_rows, kz);
-    kz = cdiv(grid_rows, kchunk);
-    if (bx > 0x7fffffffLL) return cudaErrorInvalidValue;
-    dim3 grid((unsigned)bx, (unsigned)M, (unsigned)kz), block((unsigned)bdx, (unsigned)bdy);
-    auto kern = dtype == KNN_BF16
-                    ? (vec ? bin_max_mod_kernel<KNN_BF16, 8> : bin_max_mod_kernel<KNN_BF16, 1>)
-                    : (vec ? bin_max_mod_kernel<KNN_F32, 4> : bin_max_mod_kernel<KNN_F32, 1>);
-    kern<<<grid, block, 0, st>>>(S, N, (int)L, (int)kchunk, neg, G);
+    if (cdiv(tpr, 256) > 0x7fffffffLL) return cudaErrorInvalidValue;
+    const ModShape c = mod_shape(M, grid_rows, tpr, vec ? vcols : 1);
+    dim3 grid((unsigned)cdiv(tpr, c.bdx), (unsigned)cdiv(M, c.bdz), (unsigned)c.kz),
+        block((unsigned)c.bdx, (unsigned)c.bdy, (unsigned)c.bdz);
+    auto kern = c.bdz > 1 ? mod_kernel<true>(dtype, vec) : mod_kernel<false>(dtype, vec);
+    kern<<<grid, block, 0, st>>>(S, (int)M, N, (int)L, (int)c.kchunk, neg, G);
   } else {
     const bool vec = N % vcols == 0 && (reinterpret_cast<uintptr_t>(S) & 15) == 0;
     // columns per CTA: 32 vectors per thread, or 32 columns per thread

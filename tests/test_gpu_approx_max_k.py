@@ -151,3 +151,54 @@ def test_approx_max_k_nan_comes_first(bins, dtype):
                 np.testing.assert_array_equal(i.cpu().numpy(), first)
                 np.testing.assert_array_equal(v.cpu().numpy().astype(np.float64),
                                               np.take_along_axis(Xo, first, 1))
+
+
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("M,N,L", [(1, 300_000, 8), (1, 262_144, 2064), (3, 65_536, 128),
+                                   (65, 4096, 128), (66, 4099, 128), (1000, 1024, 8), (300, 513, 40),
+                                   (67, 64, 8), (70_001, 24, 8), (5, 1000, 1)])
+def test_approx_max_k_work_split(M, N, L, dtype):
+    """How rows, grid rows and bins are shared out over threads and CTAs: many
+    chunks of one row, several rows to a CTA (the last CTA part empty), more
+    rows than one launch takes; integers, so ties keep the smaller column."""
+    ensure_built()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N + L)
+    t = torch.randint(-9, 10, (M, N), generator=g, device="cuda").float()
+    if dtype == "bf16":
+        t = t.to(torch.bfloat16)
+    T = (N + L - 1) // L
+    s = torch.full((M, T * L), -float("inf"), device="cuda")
+    s[:, :N] = t.float()
+    s = s.view(M, T, L)
+    best = s.amax(1)
+    first = (s == best[:, None, :]).float().argmax(1)
+    v, i = S.approx_max_k(t, 1, L=L, aggregate_to_topk=False)
+    assert torch.equal(v, best)
+    assert torch.equal(i.long(), first * L + torch.arange(L, device="cuda")[None, :])
+
+
+def us(f):
+    for _ in range(3):
+        f()
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    t = []
+    for _ in range(11):
+        a.record()
+        for _ in range(8):       # (of one call the host takes as long)
+            f()
+        b.record()
+        b.synchronize()
+        t.append(a.elapsed_time(b))
+    return min(t)
+
+
+def test_approx_max_k_of_many_short_rows():
+    """20,000 rows of 1024 scores take about as long as 5000 rows of 4096 (with
+    all of a CTA's threads over one row's 128 grid rows, twice as long)."""
+    ensure_built()
+    t = torch.zeros((5000, 4096), device="cuda")
+    long_rows = us(lambda: S.approx_max_k(t, 1, L=8, aggregate_to_topk=False))
+    t = t.view(20_000, 1024)
+    short_rows = us(lambda: S.approx_max_k(t, 1, L=8, aggregate_to_topk=False))
+    assert short_rows < 1.5 * long_rows
