@@ -128,3 +128,42 @@ def test_rescoring_of_a_query_per_sm_does_not_crowd():
     x, q = ints((60_000, 64), 3, -2, 3), ints((100, 64), 4, -2, 3)
     d = S.Database(x, metric="l2", dtype="bf16")
     assert us(d, q, 1024, 1024, 1) < 1.5 * us(d, q[:1], 1024, 1024, 1)
+
+
+@pytest.mark.parametrize("L", [1, 16, 32, 33, 64, 128, 129, 256, 257, 512, 513])
+def test_sorted_selection_of_many_rows(L):
+    """Many rows of few bins (a warp each up to L = 256, or 512 and K = 16),
+    with ties and rows whose bins are partly empty of finite scores."""
+    ensure_built()
+    M = 2500
+    for hi in (2, 1 << 20):
+        s = ints((M, L), L + hi, 0, hi)
+        s[::7, L // 2:] = -float("inf")
+        for K in {1, 10, 16, 17, 32, 33, 64, 65}:
+            if K > L:
+                continue
+            v, i = S.approx_max_k(s, K, L=L)
+            rv, ri = ranked(s, K)
+            assert torch.equal(v, rv)
+            assert torch.equal(i.long(), ri)
+
+
+def test_selection_of_few_bins_from_many_rows():
+    """The top K of 70,000 rows of 32 bins costs no more than twice their
+    winners alone (with a CTA to a row, 5 times)."""
+    ensure_built()
+    s = ints((70_000, 64), 9, 0, 1 << 20)
+
+    def t(agg):
+        f = lambda: S.approx_max_k(s, 4, L=32, aggregate_to_topk=agg)
+        for _ in range(3):
+            f()
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        a.record()
+        for _ in range(20):
+            f()
+        b.record()
+        b.synchronize()
+        return a.elapsed_time(b)
+
+    assert t(True) < 2 * t(False)
