@@ -746,9 +746,12 @@ cudaError_t run_k2_warp(const uint64_t* G, int64_t M, int64_t L, int K, int neg,
 // where the CTAs are about as many as a few per SM; below, they cannot crowd
 // much (1 query 47 and 49 us, 32 queries and 400 candidates 30 and 31), above, they
 // fill the chip either way (1000 queries 133.7 and 134.9; 600 queries 103 and 88).
+// (after another kernel, which starts nothing early, early_ok: 250 rows of
+// approx_max_k 1 us less)
 template <typename... KArgs, typename... Args>
-cudaError_t launch_per_query(void (*kernel)(KArgs...), int64_t M, cudaStream_t st, Args... args) {
-  if (M <= 48 || M >= 4 * device_sm_count())
+cudaError_t launch_per_query(void (*kernel)(KArgs...), int64_t M, bool early_ok, cudaStream_t st,
+                             Args... args) {
+  if (early_ok || M <= 48 || M >= 4 * device_sm_count())
     return launch_pdl(kernel, dim3((unsigned)M), dim3(256), 0, st, args...);
   kernel<<<(unsigned)M, 256, 0, st>>>(args...);
   return cudaGetLastError();
@@ -765,12 +768,13 @@ cudaError_t run_k2_select(const Src& src, int64_t M, int64_t L, int Kp, bool sor
     kern = L <= 2048   ? k2_select_kernel<Src, 8, true>
            : L <= 4096 ? k2_select_kernel<Src, 16, true>
                        : k2_select_kernel<Src, 32, true>;
-  return launch_per_query(kern, M, st, src, (int)L, Kp, sorted, out, neg, out_val, out_idx);
+  return launch_per_query(kern, M, out_val != nullptr, st, src, (int)L, Kp, sorted, out, neg,
+                          out_val, out_idx);
 }
 template <class Src, bool VEC4>
 cudaError_t run_rescore(const Src& src, int64_t M, const RescoreArgs& a, cudaStream_t st) {
   auto kern = a.L <= 1024 ? rescore_kernel<Src, 4, VEC4> : rescore_kernel<Src, 8, VEC4>;
-  return launch_per_query(kern, M, st, src, a);
+  return launch_per_query(kern, M, false, st, src, a);
 }
 
 // ---------------------------------------------------------------------------
