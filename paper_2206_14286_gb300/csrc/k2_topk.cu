@@ -739,22 +739,24 @@ cudaError_t run_k2_warp(const uint64_t* G, int64_t M, int64_t L, int K, int neg,
   return cudaGetLastError();
 }
 
-// Launches a kernel of one CTA per query that follows a contraction. Launched
-// early it saves about 2 us, but its CTAs then go where the first SMs fall free,
-// four to eight to an SM while others idle: with 100 queries, L = 1024 and 1024
-// candidates of 64 elements 90 us a search, launched in order 49. So it waits
-// where the CTAs are about as many as a few per SM; below, they cannot crowd
-// much (1 query 47 and 49 us, 32 queries and 400 candidates 30 and 31), above, they
-// fill the chip either way (1000 queries 133.7 and 134.9; 600 queries 103 and 88).
-// (after another kernel, which starts nothing early, early_ok: 250 rows of
-// approx_max_k 1 us less)
+// Launches a kernel of one CTA per query that selects (and re-ranks) Kp keys.
+// Launched early behind a contraction it saves about 2 us, but its CTAs then go
+// where the first SMs fall free, four to eight to an SM while others idle: with
+// 100 queries, L = 1024 and 1024 candidates of 64 elements 90 us a search,
+// launched in order 49. It is launched early where the CTAs are short (Kp <= 32:
+// in order the same or up to 9% longer, M = 1 to 800), few (16 queries, Kp = 256:
+// 0-12% longer; 1024 candidates of 16 queries on 200,000 rows 31% less), or so many
+// that they fill the chip either way (800 queries 0-8% longer; 450 queries, Kp = 40,
+// 128, 512: 0-3, 4-15, 4-23% less).
 template <typename... KArgs, typename... Args>
-cudaError_t launch_per_query(void (*kernel)(KArgs...), int64_t M, bool early_ok, cudaStream_t st,
+cudaError_t launch_per_query(void (*kernel)(KArgs...), int64_t M, bool early, cudaStream_t st,
                              Args... args) {
-  if (early_ok || M <= 48 || M >= 4 * device_sm_count())
-    return launch_pdl(kernel, dim3((unsigned)M), dim3(256), 0, st, args...);
+  if (early) return launch_pdl(kernel, dim3((unsigned)M), dim3(256), 0, st, args...);
   kernel<<<(unsigned)M, 256, 0, st>>>(args...);
   return cudaGetLastError();
+}
+bool early_better(int64_t M, int Kp) {
+  return Kp <= 32 || M <= 8 || (M <= 32 && Kp <= 256) || M >= 4 * device_sm_count();
 }
 
 template <class Src>
@@ -768,13 +770,14 @@ cudaError_t run_k2_select(const Src& src, int64_t M, int64_t L, int Kp, bool sor
     kern = L <= 2048   ? k2_select_kernel<Src, 8, true>
            : L <= 4096 ? k2_select_kernel<Src, 16, true>
                        : k2_select_kernel<Src, 32, true>;
-  return launch_per_query(kern, M, out_val != nullptr, st, src, (int)L, Kp, sorted, out, neg,
-                          out_val, out_idx);
+  // (values and indices follow kernels that let nothing start early: no crowding)
+  return launch_per_query(kern, M, out_val || early_better(M, Kp), st, src, (int)L, Kp, sorted,
+                          out, neg, out_val, out_idx);
 }
 template <class Src, bool VEC4>
 cudaError_t run_rescore(const Src& src, int64_t M, const RescoreArgs& a, cudaStream_t st) {
   auto kern = a.L <= 1024 ? rescore_kernel<Src, 4, VEC4> : rescore_kernel<Src, 8, VEC4>;
-  return launch_per_query(kern, M, false, st, src, a);
+  return launch_per_query(kern, M, early_better(M, a.Kp), st, src, a);
 }
 
 // ---------------------------------------------------------------------------

@@ -105,7 +105,7 @@ def test_selection_of_more_than_1024_candidates_stays_a_selection():
     assert us(d, q, 205, 8192, 5) < 2.2 * us(d, q, 128, 8192, 8)
 
 
-@pytest.mark.parametrize("M", [47, 48, 49, 151, 152, 607, 608, 609])
+@pytest.mark.parametrize("M", [8, 9, 32, 33, 47, 48, 49, 151, 152, 607, 608, 609])
 def test_rescored_search_of_a_few_queries_per_sm(M):
     """The numbers of queries around which the rescoring's launch changes."""
     ensure_built()
@@ -113,7 +113,7 @@ def test_rescored_search_of_a_few_queries_per_sm(M):
         x, q = ints((N, 24), N + M, -2, 3), ints((M, 24), M, -2, 3)
         d = S.Database(x, metric="ip", dtype="bf16")
         s = q @ x.t()
-        for K, r in ((10, 2), (100, 8)):
+        for K, r in ((10, 2), (33, 1), (257, 1), (100, 8)):
             val, idx = d.search(q, K, L=N, rerank=r)
             rv, ri = ranked(s, K)
             assert torch.equal(idx.long(), ri)
