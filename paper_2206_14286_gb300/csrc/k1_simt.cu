@@ -260,12 +260,16 @@ cudaError_t launch_simt(const K1Plan& p, const float* X, const float* hnorm, con
   // 468, 293 and 290).
   const int64_t sms = device_sm_count();
   if (blocks <= sms) smem = 96 * 1024;
-  // Up to two to an SM with many of them short (the last of few splits): launched
-  // in order the short ones share SMs with the others (1000 queries on 3000 x 768
-  // rows, L = 1024, 3 tiles in splits of 2 and 1: 178 and 139 us). Even ones gain
-  // from the early start (65 queries on 16,384 x 128 rows: 24 and 27 us).
-  const bool in_order = blocks > sms && blocks < 2 * sms &&
-                        4 * (p.nsplits * p.tiles_per_split - p.ntiles) >= p.ntiles;
+  // Up to two to an SM, with many of them short (the last of few splits) or all of
+  // them long: launched in order the short ones share SMs with the others (1000
+  // queries on 3000 x 768 rows, L = 1024, 3 tiles in splits of 2 and 1: 178 and 139
+  // us), and those alone on an SM are worth more than the early start (256 queries on
+  // 9000 x 2000 rows, L = 2000: 479 and 380). Short even ones gain from the early
+  // start (65 queries on 16,384 x 128 rows: 24 and 27 us).
+  const bool in_order =
+      blocks > sms && blocks < 2 * sms &&
+      (4 * (p.nsplits * p.tiles_per_split - p.ntiles) >= p.ntiles ||
+       p.tiles_per_split * p.pitch >= 1536);
   if (smem > 0) {
     cudaError_t e =
         cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
