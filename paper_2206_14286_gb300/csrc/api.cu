@@ -104,12 +104,14 @@ int64_t plan_bins(int64_t N, int K, double r, int round_to) {
 }
 
 // Tile shape of each K1 variant (BQ = 0: the row length is not supported).
-// scores: the exact search's kernel, one bin per row.
-void k1_tile(int dtype, int D, int64_t M, bool scores, int* BW, int* BQ) {
+// scores: the exact search's kernel, one bin per row of N; its tiles of 128 rows
+// are halved where that many leave half of the SMs without one (333 queries on
+// 3000 x 4096 rows, 72 tiles: 513 us a call, halved 360; 128 queries 491 and 306).
+void k1_tile(int dtype, int D, int64_t N, int64_t M, bool scores, int* BW, int* BQ) {
   dtype = stored_dtype(dtype);
   if (dtype == KNN_F32) {
     *BQ = M <= 64 ? 64 : 128;
-    *BW = scores && *BQ == 128 ? 128 : 64;
+    *BW = scores && *BQ == 128 && 2 * cdiv(N, 128) * cdiv(M, 128) > device_sm_count() ? 128 : 64;
   } else {
     *BW = 128;
     const int maxq = k1_tc_query_tile(dtype, D);
@@ -135,7 +137,7 @@ K1Plan make_plan(int64_t N, int64_t M, int64_t L, int D, int metric, int dtype,
   p.pitch = (int)round_up(D, 16);
   p.metric = metric;
   p.dtype = stored_dtype(dtype);  // KNN_E4M3_T runs here as KNN_E4M3 (all scales equal)
-  k1_tile(dtype, D, M, force_splits > 0, &p.BW, &p.BQ);
+  k1_tile(dtype, D, N, M, force_splits > 0, &p.BW, &p.BQ);
   if (p.BQ == 0) return p;
   p.g = L < p.BW ? (int)(p.BW / L) : 1;
   p.Lk = (int64_t)p.g * L;
@@ -453,7 +455,7 @@ knn_status layout_exact(const SearchArgs& a, ExactLayout* s) {
   knn_status st = check_sizes(a.N, a.D, a.dtype, a.metric, a.M, a.K);
   if (st != KNN_OK) return st;
   int BW, BQ;
-  k1_tile(a.dtype, a.D, a.M, true, &BW, &BQ);
+  k1_tile(a.dtype, a.D, a.N, a.M, true, &BW, &BQ);
   if (BQ == 0) return KNN_EUNSUPPORTED;
   int64_t mq = a.M > 0 ? a.M : 1;
   int64_t nc = (kExactPartialBudget / mq) / BW * BW;

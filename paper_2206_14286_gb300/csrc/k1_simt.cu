@@ -26,7 +26,8 @@
 //
 // kScores: an exact search's chunk, one bin per row: the scores themselves are
 // written (4 bytes each), no state and no merge; 128 rows per tile (TB = 8, with
-// 128 queries), which halves the shared-memory operand reads per product.
+// 128 queries and tiles for half of the SMs or more), which halves the
+// shared-memory operand reads per product.
 #include "common.cuh"
 #include "kernels.h"
 
@@ -289,15 +290,16 @@ cudaError_t launch_simt_tile(const K1Plan& p, const float* X, const float* hnorm
   if (out.keys64)
     return p.BQ == 64 ? launch_simt<METRIC, 4, 4, false>(p, X, hnorm, Qp, out.v, blocks, st)
                       : launch_simt<METRIC, 8, 4, false>(p, X, hnorm, Qp, out.v, blocks, st);
-  return p.BQ == 64 ? launch_simt<METRIC, 4, 4, true>(p, X, hnorm, Qp, out.v, blocks, st)
-                    : launch_simt<METRIC, 8, 8, true>(p, X, hnorm, Qp, out.v, blocks, st);
+  return p.BQ == 64   ? launch_simt<METRIC, 4, 4, true>(p, X, hnorm, Qp, out.v, blocks, st)
+         : p.BW == 64 ? launch_simt<METRIC, 8, 4, true>(p, X, hnorm, Qp, out.v, blocks, st)
+                      : launch_simt<METRIC, 8, 8, true>(p, X, hnorm, Qp, out.v, blocks, st);
 }
 }  // namespace
 
 cudaError_t launch_k1_simt(const K1Plan& p, const float* X, const float* hnorm, const float* Qp,
                            Partials out, cudaStream_t st) {
-  const int bw = !out.keys64 && p.BQ == 128 ? 128 : 64;
-  if (p.BW != bw || (p.BQ != 64 && p.BQ != 128) || (p.pitch % BD) != 0)
+  if ((p.BW != 64 && (p.BW != 128 || out.keys64 || p.BQ != 128)) ||
+      (p.BQ != 64 && p.BQ != 128) || (p.pitch % BD) != 0)
     return cudaErrorInvalidValue;
   if (!out.keys64 && p.ntiles != 1) return cudaErrorInvalidValue;
   int64_t blocks = p.nsplits * p.nstrips * p.nqtiles;

@@ -84,3 +84,41 @@ def test_partial_reduce_f32_order(M, N, L):
     first = (p == best[:, None, :]).to(torch.uint8).argmax(1) * L + torch.arange(L, device="cuda")
     assert torch.equal(V.double(), best)
     assert torch.equal(A.long(), first)
+
+
+@pytest.mark.parametrize("M,N", [(65, 9728), (65, 9729), (333, 3000), (333, 3300), (1000, 1216),
+                                 (1000, 1217), (129, 100), (4865, 65), (9729, 65)])
+def test_exact_search_tile_sizes(M, N):
+    """FP32 tiles of 128 rows, or of 64 where the larger would leave half of the
+    SMs without one."""
+    ensure_built()
+    x, q = rows(N, 20, M), rows(M, 20, N)
+    d = S.Database(x, metric="ip", dtype="f32")
+    val, idx = d.search_exact(q, 10)
+    v, a = ranked(q @ x.t(), 10)
+    assert torch.equal(idx.long(), a)
+    assert torch.equal(val, v)
+
+
+def test_exact_search_of_few_rows_is_shared_out():
+    """128 queries on 3000 long rows, in tiles of 128 x 64, take up to 1.65 times
+    as long as 64 in tiles of 64 x 64 (with 24 tiles of 128 x 128, twice)."""
+    ensure_built()
+    x, q = rows(3000, 4096, 1), rows(128, 4096, 2)
+    d = S.Database(x, metric="ip", dtype="f32")
+
+    def us(q):
+        for _ in range(3):
+            d.search_exact(q, 10)
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        t = []
+        for _ in range(9):
+            a.record()
+            for _ in range(4):
+                d.search_exact(q, 10)
+            b.record()
+            b.synchronize()
+            t.append(a.elapsed_time(b))
+        return min(t)
+
+    assert us(q) < 1.65 * us(q[:64])
