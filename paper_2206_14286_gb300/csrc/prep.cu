@@ -72,15 +72,17 @@ __device__ __forceinline__ void add_square(Triple& a, float v) {
 }
 
 // Magnitudes for which the pairs behave (anything else, zero rows too, takes
-// the FP64 way). square_range: squares and their error terms neither overflow
-// nor lose bits that matter against the sum of the row's squares. unit_range,
-// for the inverse norm: its square, at least 2^(-2 kUnitHi) / kMaxD, is also
+// the FP64 way). square_range, for the half norm: squares and their error terms
+// neither overflow nor lose bits that matter against the sum of the row's
+// squares: an element's square and its error term lose up to 2^-149, 2^-137 for
+// the longest row, 2^-37 of the largest element's square. unit_range, for the
+// inverse norm: its square, at least 2^(-2 kUnitHi) / kMaxD, is also
 // held exactly as two FP32 numbers: its last bit, 2^-48 of it, is no smaller
 // than FP32's smallest number, 2^-149. (With elements up to 2^50 that bit was
 // lost, and 1 / |x| was off by up to 2^-41 at D = 1024.)
 constexpr int kUnitHi = 40;
 static_assert(2 * kUnitHi + 48 <= 149 - 12 && kMaxD <= 1 << 12, "1 / |x|^2 loses bits");
-__device__ __forceinline__ bool square_range(float mx) { return mx >= 0x1p-40f && mx <= 0x1p50f; }
+__device__ __forceinline__ bool square_range(float mx) { return mx >= 0x1p-50f && mx <= 0x1p50f; }
 __device__ __forceinline__ bool unit_range(float mx) {
   return mx >= 0x1p-40f && mx <= (float)(1ll << kUnitHi);
 }
@@ -516,13 +518,15 @@ prep_rows_kernel(const float* __restrict__ x, int64_t rows, int D, int pitch, in
   if (!COS && out_hnorm) {
     // half the sum, rounded once; the FP64 sum where the pair's error bound
     // (2^-36 of the sum with 32 elements per lane, 2^-32 with 128) leaves the
-    // rounding open
+    // rounding open. A row of zeros is 0 (50,000 x 257 rows of zeros or of
+    // elements at 2^-45 took 122 us in both, 79 in FP64 alone)
     h2 = group_sum<G>(h2);
     smx = group_max<G>(smx);
     const float m = __fmul_rn(h2.h, VPL > 0 ? 0x1p-35f : 0x1p-31f);
     const float up = __fadd_rn(h2.h, __fadd_rn(h2.l, m)), dn = __fadd_rn(h2.h, __fsub_rn(h2.l, m));
-    const bool open = !(up == dn && square_range(smx));
-    float hn = 0.5f * up;
+    const bool zero = smx == 0.0f && h2.h == 0.0f;  // (a NaN is in h2.h only)
+    const bool open = !zero && !(up == dn && square_range(smx));
+    float hn = zero ? 0.0f : 0.5f * up;
     if (group_any<32>(open && live)) {
       double a = 0.0;
       if (live) {

@@ -147,3 +147,49 @@ def test_prepare_bits_at_the_ends_of_the_paired_range(D):
     d = S.Database(torch.from_numpy(X).cuda(), metric="l2", dtype="f32")
     X64 = X.astype(np.float64)
     np.testing.assert_array_equal(d.hnorm.cpu().numpy(), (0.5 * (X64 * X64).sum(1)).astype(np.float32))
+
+
+@pytest.mark.parametrize("D", [64, 257, 1024, 1500, 4096])
+def test_half_norms_of_small_rows(D):
+    """L2 half norms of rows of zeros (of either sign, with a NaN or not) and
+    around the lower end of the range that paired FP32 handles (2^-50)."""
+    ensure_built()
+    g = np.random.Generator(np.random.PCG64(D + 1))
+    tops = [2.0 ** e for e in (-70, -52, -51, -50, -49, -45)]
+    tops += [np.nextafter(np.float32(2.0 ** -50), np.float32(0.0))]
+    X = g.uniform(0.25, 1.0, (32 * len(tops), D)) * np.repeat(tops, 32)[:, None]
+    X[:, ::3] *= 2.0 ** -12                     # squares that lose bits
+    X[:, 0] = np.repeat(tops, 32)
+    X = X.astype(np.float32)
+    X[5] = 0.0
+    X[6] = -0.0
+    X[7] = 0.0
+    X[7, D // 2] = np.nan
+    X[8] = 0.0
+    X[8, D - 1] = np.float32(2.0 ** -140)
+    d = S.Database(torch.from_numpy(X).cuda(), metric="l2", dtype="f32")
+    X64 = X.astype(np.float64)
+    h = (0.5 * (X64 * X64).sum(1)).astype(np.float32)
+    np.testing.assert_array_equal(d.hnorm.cpu().numpy(), h)
+
+
+def test_rows_of_zeros_cost_no_more_than_others():
+    """(in FP64 beside the paired FP32, 3 times as much)"""
+    ensure_built()
+
+    def ms(x):
+        for _ in range(3):
+            S.Database(x, metric="l2", dtype="f32")
+        a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        t = []
+        for _ in range(9):
+            a.record()
+            for _ in range(8):
+                S.Database(x, metric="l2", dtype="f32")
+            b.record()
+            b.synchronize()
+            t.append(a.elapsed_time(b))
+        return min(t)
+
+    x = torch.randn((50_000, 257), device="cuda")
+    assert ms(torch.zeros_like(x)) < 1.5 * ms(x)
