@@ -476,8 +476,10 @@ knn_status layout_exact(const SearchArgs& a, ExactLayout* s) {
   o += al((size_t)s->plan.M * (size_t)round_up(s->plan.Lk, 4) * 4);
   s->off_run = o;
   o += al((size_t)a.M * a.K * 8);
+  // up to kExactMaxK two running sets in turn and the blocks' keys; larger K
+  // updates one set in place
   s->off_run2 = o;
-  o += al((size_t)a.M * a.K * 8);
+  if (a.K <= kExactMaxK) o += al((size_t)a.M * a.K * 8);
   s->off_cand = o;
   if (a.K <= kExactMaxK) o += al(exact_cand_bytes(a.M, nc, a.K));
   s->total = o > kAlign ? o : kAlign;

@@ -4,8 +4,10 @@ import numpy as np
 import pytest
 import torch
 
+from paper_2206_14286_gb300 import _lib
 from paper_2206_14286_gb300 import build as B
 from paper_2206_14286_gb300 import search as S
+from paper_2206_14286_gb300._lib import DTYPE, METRIC
 
 
 def database(N=100_000, D=64):
@@ -36,3 +38,12 @@ def test_plans_are_bounded():
     for M in range(1, 600):
         d._search_plan(M, 10, 1000, 0.95, 2, "mod")
         assert len(d._plans) <= 256
+
+
+def test_exact_workspace_of_large_k_holds_one_running_set():
+    """Beyond 1024 results the running set is updated in place: 500 more of them
+    for 128 queries are 500 x 128 keys."""
+    B.build()
+    ws = [_lib.get().knn_search_exact_workspace(100_000, 64, DTYPE["f32"], METRIC["l2"], 128, K)
+          for K in (1500, 2000)]
+    assert ws[1] - ws[0] == 500 * 128 * 8
