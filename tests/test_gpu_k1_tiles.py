@@ -139,3 +139,88 @@ def test_few_bins_do_not_queue_for_their_keys():
     q = torch.randn((64, 64), generator=g, device="cuda")
     d = S.Database(x, metric="ip", dtype="bf16")
     assert us(lambda: d.partial_reduce(q, 3)) < 1.6 * us(lambda: d.partial_reduce(q, 20))
+
+
+def schedule(nqt, steps, sms):
+    """(tiles per CTA, steps per CTA) of the tensor-core kernel's host schedule."""
+    first = (nqt + sms - 1) // sms
+    best = None
+    for kq in range(first, min(nqt, first + 16) + 1):
+        groups = (nqt + kq - 1) // kq
+        if groups > sms:
+            continue
+        parts = min(sms // groups, steps)
+        spp = (steps + parts - 1) // parts
+        if best is None or kq * (spp + 1) < best[0]:
+            best = (kq * (spp + 1), kq, spp)
+    return best[1:]
+
+
+@pytest.mark.parametrize("bins", ["mod", "contiguous"])
+def test_l2_half_norms_of_several_tiles_per_cta(bins):
+    """A CTA that takes several query tiles in turn over its rows starts the
+    rows' half norms again with each, while the next tile's are already on
+    their way, and (contiguous bins) the first bin of its rows."""
+    ensure_built()
+    D, M = 64, 3339
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    odd = 0
+    for N, L in ((100_000, 605), (91_000, 333)):
+        T, r = N // L, N % L
+        up = lambda a, b: (a + b - 1) // b
+        steps = (up(r, 16) * up(T + 1, 16) + up(L - r, 16) * up(T, 16) if bins == "mod"
+                 else up(N, 256))
+        two, one = schedule(up(M, 256), steps, sms), schedule(up(M, 128), steps, sms)
+        factor = 1.1 if bins == "mod" else 1.5
+        kq, spp = one if factor * one[0] * (one[1] + 1) < 2.0 * two[0] * (two[1] + 1) else two
+        assert kq >= 2
+        odd += spp % 2
+        g = torch.Generator(device="cuda")
+        g.manual_seed(L)
+        x = torch.randint(-2, 3, (N, D), generator=g, device="cuda").float()
+        q = torch.randint(-2, 3, (M, D), generator=g, device="cuda").float()
+        d = S.Database(x, metric="l2", dtype="bf16")
+        V, A = d.partial_reduce(q, L, bins=bins)
+        S.sync_status()
+        s = q @ x.t() - 0.5 * (x * x).sum(1)[None, :]
+        best, first = bin_winners(s, L, bins)
+        assert torch.equal(V, best)
+        assert torch.equal(A.long(), first)
+        del s, best, first
+    assert odd          # an odd number of steps per tile, too
+
+
+def bin_winners(s, L, bins):
+    """(best score, first row that has it) of each bin, M x L."""
+    M, N = s.shape
+    j = torch.arange(N, device=s.device)
+    b = bin_of(N, L, bins)[None, :].expand(M, N)
+    best = torch.full((M, L), -float("inf"), device=s.device).scatter_reduce(1, b, s, "amax")
+    at = torch.where(s == best.gather(1, b), j[None, :], N)
+    first = torch.full((M, L), N, device=s.device).scatter_reduce(1, b, at, "amin")
+    return best, first
+
+
+@pytest.mark.parametrize("dtype,metric", [("bf16", "ip"), ("bf16", "l2"), ("e4m3t", "ip")])
+@pytest.mark.parametrize("M", [1, 128, 129, 333])
+@pytest.mark.parametrize("N,L", [(40_011, 3), (40_011, 20), (40_011, 605), (4097, 16), (300, 77)])
+def test_partial_reduce_ties_keep_the_smaller_row(dtype, metric, M, N, L):
+    """Integers, whose scores are exact and mostly tie: through virtual bins,
+    both grids, accumulators that take alternate steps and the search for a
+    run's position."""
+    ensure_built()
+    g = torch.Generator(device="cuda")
+    g.manual_seed(N + L + M)
+    x = torch.randint(-2, 3, (N, 24), generator=g, device="cuda").float()
+    q = torch.randint(-2, 3, (M, 24), generator=g, device="cuda").float()
+    if dtype == "e4m3t":          # scales 1: the codes are the values
+        x[:, 0], q[:, 0] = 448.0, 448.0
+    s = q @ x.t()
+    if metric == "l2":
+        s = s - 0.5 * (x * x).sum(1)[None, :]
+    d = S.Database(x, metric=metric, dtype=dtype)
+    for bins in ("mod", "contiguous"):
+        V, A = d.partial_reduce(q, L, bins=bins)
+        best, first = bin_winners(s, L, bins)
+        assert torch.equal(V, best)
+        assert torch.equal(A.long(), first)
