@@ -154,7 +154,7 @@ K1Plan make_plan(int64_t N, int64_t M, int64_t L, int D, int metric, int dtype,
     if (dtype == KNN_F32 && sms > 0) {
       // SIMT CTAs run two per SM: the split count with the least
       // (waves of 2 * sms CTAs) x (tiles per CTA), the smallest on ties,
-      // which also keeps the per-split partials no larger than needed
+      // which also makes the fewest merges into a bin's key
       // (for each number of tiles per CTA, the smallest split count with it: the
       // others only add CTAs)
       const int64_t wave = 2 * sms;
