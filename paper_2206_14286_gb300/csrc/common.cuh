@@ -39,6 +39,19 @@ cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   return cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
+// ---------------------------------------------------------------------------
+// Allows a kernel dynamic shared memory. The allowance belongs to the kernel, and
+// any thread's launch of it may follow: where the launches' sizes vary, all of
+// them allow the same largest size. (Each allowing its own, a thread that
+// launched with less could take the allowance back between another's setting
+// and its launch, which was then refused.)
+// ---------------------------------------------------------------------------
+constexpr int kMaxDynamicSmem = 227 * 1024;  // without static shared memory
+template <class Kernel>
+cudaError_t allow_dynamic_smem(Kernel kernel, int largest = kMaxDynamicSmem) {
+  return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, largest);
+}
+
 constexpr int kMaxK = 4096;       // largest K (and K') a search accepts
 constexpr int kMaxD = 4096;       // largest row length
 constexpr uint32_t kNegInfBits = 0xff800000u;

@@ -260,7 +260,8 @@ cudaError_t launch_simt(const K1Plan& p, const float* X, const float* hnorm, con
   // L2, 144 CTAs: 93 us a call without, 65 launched in order, 61 so; 4096 elements
   // 468, 293 and 290).
   const int64_t sms = device_sm_count();
-  if (blocks <= sms) smem = 96 * 1024;
+  constexpr int kOwnSm = 96 * 1024;
+  if (blocks <= sms) smem = kOwnSm;
   // Up to two to an SM, with many of them short (the last of few splits) or all of
   // them long: launched in order the short ones share SMs with the others (1000
   // queries on 3000 x 768 rows, L = 1024, 3 tiles in splits of 2 and 1: 178 and 139
@@ -272,8 +273,7 @@ cudaError_t launch_simt(const K1Plan& p, const float* X, const float* hnorm, con
       (4 * (p.nsplits * p.tiles_per_split - p.ntiles) >= p.ntiles ||
        p.tiles_per_split * p.pitch >= 1536);
   if (smem > 0) {
-    cudaError_t e =
-        cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(kern, kOwnSm);
     if (e != cudaSuccess) return e;
   }
   unsigned long long* G = reinterpret_cast<unsigned long long*>(v);

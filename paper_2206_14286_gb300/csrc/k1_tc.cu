@@ -348,7 +348,7 @@ template <int DT, int METRIC, int BQ>
 cudaError_t launch_variant(const CUtensorMap& mx, const CUtensorMap& mq, const TcArgs& a,
                            size_t smem, int64_t blocks, cudaStream_t st) {
   auto kern = k1_tc_kernel<DT, METRIC, BQ>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_dynamic_smem(kern);
   if (e != cudaSuccess) return e;
   kern<<<(unsigned)blocks, kThreads, smem, st>>>(mx, mq, a);
   return cudaGetLastError();

@@ -1081,7 +1081,7 @@ cudaError_t launch_tcs(const CUtensorMap (&mx)[2], const CUtensorMap& mq, const 
   if (e != cudaSuccess) return e;
   if ((int64_t)round_up(fa.numRegs, 8) * kThreadsS < 128 * kCtrlRegsS + 512 * kEpiRegsS)
     return cudaErrorNotSupported;
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  e = allow_dynamic_smem(kern);
   if (e != cudaSuccess) return e;
   if constexpr (BM == kBinsRun) {
     // Contiguous bins: a plain launch. Started early behind the query prep,

@@ -258,10 +258,10 @@ cudaError_t launch_k3(int64_t M, int D, int metric, const uint64_t* cand, int Kp
                          N, out_val, out_idx, st);
   const int P2 = next_pow2(Kp > K ? Kp : K);
   const size_t smem = (size_t)P2 * sizeof(uint64_t);
-  if (smem > 200 * 1024) return cudaErrorInvalidValue;
+  constexpr int kLargest = 200 * 1024;
+  if (smem > kLargest) return cudaErrorInvalidValue;
   if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(k3_rerank_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_dynamic_smem(k3_rerank_kernel, kLargest);
     if (e != cudaSuccess) return e;
   }
   k3_rerank_kernel<<<(unsigned)M, 256, smem, st>>>(cand, Kp, K, P2, D, metric, qf32, q_stride,
